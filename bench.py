@@ -88,6 +88,9 @@ KNOWN_TRAFFIC: dict[str, float] = {
     # the same kernel waiting for its TMEM stores before every scoring:
     # read 689,644,885 + write 7,989,676,288 (mean of 3 launches)
     "22e4d6d25dce": 8679321173.0,
+    # walkers with paired FP32 and running addresses:
+    # read 708,970,496 + write 8,006,513,664 (mean of 2 launches)
+    "686a90346174": 8715484160.0,
 }
 KERNEL_SOURCES = ("fuse_tile.cuh", "fuse_metrics.cu", "metric_q.cuh", "tmem.cuh")
 

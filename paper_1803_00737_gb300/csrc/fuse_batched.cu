@@ -1,0 +1,186 @@
+// Batched fused forward: the persistent kernel fed by a device-side work queue.
+#include <algorithm>
+
+#include "fuse_tile.cuh"
+#include "launch.h"
+
+namespace dwtfuse {
+
+constexpr int kBatchNarrowBands = 4;  // instance for entries of at most 4 bands
+constexpr int kSceneBytes = (int)((sizeof(SceneArgs) + 15) / 16 * 16);
+
+// Threads per CTA (two CTAs per SM), walker mode and shared memory (per warp, a
+// copy of its item's scene) of an instance.  Entries of at most 4 bands:
+// uint8 20 warps per SM at up to 96 registers (24 uneven scenes of 3-8 bands,
+// 256..4096 px: 719 us a call against 730 with 16 warps at 128), float 16
+// warps with the next row's inputs loaded ahead (forward + backward of
+// 8 x 4096^2 x 4: 1086 us a pass against 1129 with 20 warps, where that
+// spills, and 1101 with 16 and no loads ahead).
+template <typename T, int MAXB>
+struct BatchShape {
+    static constexpr bool kNarrow = MAXB <= kBatchNarrowBands, kFloat = sizeof(T) == 4;
+    static constexpr int kThreads = kNarrow && !kFloat ? 320 : 256;
+    static constexpr int kMode = kNarrow && kFloat ? kAheadPan | kAheadMs : 0;
+    static constexpr int kSmem = kThreads / 32 * kSceneBytes;
+};
+
+extern __shared__ __align__(16) unsigned char batch_smem[];
+
+// One item of a scene with NB bands: the scene is the warp's shared-memory
+// copy (in the kernel's parameter block it would be read at run-time offsets
+// and its members held in registers).  A function of its own, not inlined:
+// each of an instance's bodies gets its own register allocation (all inlined
+// in one kernel they spilled up to 0.5 KB a thread).
+template <typename T, int WAV, int NB, int LAY, int MODE>
+static __device__ __noinline__ void batch_body(int x0, int m_s, int m_e) {
+    const SceneArgs &s = *reinterpret_cast<const SceneArgs *>(batch_smem + (threadIdx.x >> 5) * kSceneBytes);
+    direct_item<T, WAV, NB, LAY, MODE>(s, x0, m_s, m_e, 0, threadIdx.x & 31);
+}
+
+// Batched: every warp pulls the next item index from `queue[0]`; item ranges
+// of the scenes are given by the prefix sums item_start[].  A warp whose
+// scene table entry fails its checks records DWTFUSE_EDEVICE in status[0].
+// An instance serves one input type and at most MAXB bands per entry.
+template <typename T, int MAXB>
+__global__ void __launch_bounds__(BatchShape<T, MAXB>::kThreads, 2)
+fuse_batched_kernel(const __grid_constant__ BatchTable t, unsigned long long *queue, int *status) {
+    constexpr int M = BatchShape<T, MAXB>::kMode;
+    uint32_t *copy = reinterpret_cast<uint32_t *>(batch_smem + (threadIdx.x >> 5) * kSceneBytes);
+    const int lane = threadIdx.x & 31;
+    const unsigned long long total = (unsigned long long)t.item_start[t.n];
+    int have = -1;  // scene the warp's copy holds
+    for (;;) {
+        unsigned long long it = 0;
+        if (lane == 0) it = atomicAdd(queue, 1ull);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= total) break;
+        int lo = 0, hi = t.n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if ((unsigned long long)t.item_start[mid] <= it) lo = mid; else hi = mid - 1;
+        }
+        const SceneArgs &s = t.scenes[lo];
+        if (s.bands < 1 || s.bands > MAXB || (s.in_f32 != 0) != (sizeof(T) == 4)) {
+            if (lane == 0) atomicCAS(status, 0, 7);
+            continue;
+        }
+        if (have != lo) {
+            __syncwarp();  // every lane is done with the previous scene
+            const uint32_t *src = reinterpret_cast<const uint32_t *>(&s);
+            for (int k = lane; k < (int)(sizeof(SceneArgs) / 4); k += 32) copy[k] = src[k];
+            have = lo;
+            __syncwarp();
+        }
+        const int64_t local = (int64_t)(it - (unsigned long long)t.item_start[lo]);
+        const int64_t sx = local % t.strips_x[lo], sy = local / t.strips_x[lo];
+        const int x0 = (int)(sx * kWarpCols), m_s = s.m_lo + (int)(sy * t.R), m_e = min(m_s + t.R, s.m_hi);
+#define DWTFUSE_CASE(NBV)                                                      \
+    case NBV:                                                                  \
+        if constexpr (NBV <= MAXB) {                                           \
+            if (s.wavelet) {                                                   \
+                if (s.a4) batch_body<T, 1, NBV, kVec, M>(x0, m_s, m_e);           \
+                else if (s.alt) batch_body<T, 1, NBV, kShift, M>(x0, m_s, m_e);   \
+                else batch_body<T, 1, NBV, kPairs, M>(x0, m_s, m_e);              \
+            } else {                                                           \
+                if (s.a4) batch_body<T, 0, NBV, kVec, M>(x0, m_s, m_e);           \
+                else if (s.alt) batch_body<T, 0, NBV, kShift, M>(x0, m_s, m_e);   \
+                else batch_body<T, 0, NBV, kPairs, M>(x0, m_s, m_e);              \
+            }                                                                  \
+        }                                                                      \
+        break;
+        switch (s.bands) {
+            DWTFUSE_CASE(1) DWTFUSE_CASE(2) DWTFUSE_CASE(3) DWTFUSE_CASE(4)
+            DWTFUSE_CASE(5) DWTFUSE_CASE(6) DWTFUSE_CASE(7) DWTFUSE_CASE(8)
+            default: break;
+        }
+#undef DWTFUSE_CASE
+    }
+}
+
+namespace {
+
+// Launches one instance over table t (entries of one input type and width
+// class).  clear: bytes of the queue word(s) to zero first (the queue counter
+// and status word, or only the counter so that a status an earlier launch of
+// the same call recorded survives).
+struct BatchFn {
+    void *fn;
+    int threads, smem;
+};
+template <typename T, int MAXB>
+BatchFn batch_fn() {
+    return {reinterpret_cast<void *>(&fuse_batched_kernel<T, MAXB>), BatchShape<T, MAXB>::kThreads,
+            BatchShape<T, MAXB>::kSmem};
+}
+
+cudaError_t launch_table(const BatchTable &t, unsigned long long *queue, int *status, int blocks_per_sm,
+                         size_t clear, cudaStream_t stream) {
+    const bool f32 = t.scenes[0].in_f32 != 0, narrow = t.scenes[0].bands <= kBatchNarrowBands;
+    const BatchFn k = f32 ? (narrow ? batch_fn<float, kBatchNarrowBands>() : batch_fn<float, kBatchMaxBands>())
+                          : (narrow ? batch_fn<uint8_t, kBatchNarrowBands>() : batch_fn<uint8_t, kBatchMaxBands>());
+    void *fn = k.fn;
+    const int threads = k.threads, smem = k.smem;
+    int occ = 0;
+    cudaError_t e = resident_blocks_smem(fn, threads, smem, &occ);
+    if (e != cudaSuccess) return e;
+    if (blocks_per_sm > 0 && blocks_per_sm < occ) occ = blocks_per_sm;
+    int sms = 0;
+    e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(queue, 0, clear, stream);
+    if (e != cudaSuccess) return e;
+    const int64_t total = t.item_start[t.n];
+    const int64_t need = (total + threads / 32 - 1) / (threads / 32);
+    const int64_t cap = (int64_t)sms * occ;
+    const unsigned grid = (unsigned)(need < cap ? need : cap);
+    if (grid == 0) return cudaSuccess;
+    void *args[] = {const_cast<BatchTable *>(&t), &queue, &status};
+    return cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, (size_t)smem, stream);
+}
+
+// The entries of t of input type f32 and width class narrow (at most
+// kBatchNarrowBands bands or more), those of one body (bands, wavelet, row
+// layout) together: warps of an SM work on neighbouring items, so they run one
+// or two bodies at a time and share their instructions (24 uneven scenes in
+// the caller's order: 768 us, instruction fetch 1.9 of 12 stall cycles per
+// issue; sorted 719 us).
+void split_table(const BatchTable &t, bool f32, bool narrow, BatchTable *o) {
+    int order[kMaxScenes], m = 0;
+    for (int i = 0; i < t.n; ++i)
+        if ((t.scenes[i].in_f32 != 0) == f32 && (t.scenes[i].bands <= kBatchNarrowBands) == narrow) order[m++] = i;
+    auto body = [&](int i) {
+        return (t.scenes[i].bands * 2 + t.scenes[i].wavelet) * 3 + row_layout(t.scenes[i].a4, t.scenes[i].alt);
+    };
+    std::stable_sort(order, order + m, [&](int a, int b) { return body(a) > body(b); });
+    o->n = m;
+    o->R = t.R;
+    o->item_start[0] = 0;
+    for (int j = 0; j < m; ++j) {
+        const int i = order[j];
+        o->scenes[j] = t.scenes[i];
+        o->strips_x[j] = t.strips_x[i];
+        o->item_start[j + 1] = o->item_start[j] + (t.item_start[i + 1] - t.item_start[i]);
+    }
+}
+
+}  // namespace
+
+// One launch per input type and width class in the table, the wide ones first.
+cudaError_t launch_fuse_batched(const BatchTable &t, unsigned long long *queue, int *status,
+                                int blocks_per_sm, cudaStream_t stream) {
+    int count[2][2] = {};
+    for (int i = 0; i < t.n; ++i) ++count[t.scenes[i].in_f32 != 0][t.scenes[i].bands <= kBatchNarrowBands];
+    static thread_local BatchTable part;
+    size_t clear = kQueueBytes;
+    for (int kind = 0; kind < 4; ++kind) {
+        const bool narrow = kind >> 1, f32 = kind & 1;
+        if (count[f32][narrow] == 0) continue;
+        split_table(t, f32, narrow, &part);
+        const cudaError_t e = launch_table(part, queue, status, blocks_per_sm, clear, stream);
+        if (e != cudaSuccess) return e;
+        clear = sizeof(unsigned long long);
+    }
+    return cudaSuccess;
+}
+
+}  // namespace dwtfuse

@@ -56,64 +56,6 @@ __device__ __forceinline__ void pair_bands(int p, int &b, int &c) {
     c = b + 1 + p;
 }
 
-// Band b of MS row m: parks its uint8 words of PAN rows 2m, 2m+1 in tile slot
-// r (of SR) and its MS reference word, and writes the fused pixels.
-template <int NB, int SR>
-__device__ __forceinline__ void metric_band(const SceneArgs &s, const LaneCols &c, uint32_t *tile, uint32_t *rep,
-                                            int lane, int r, bool a4, bool alt, int b, int64_t m,
-                                            const float *v0, const float *v1, float mn, float mn1) {
-    const uint32_t w0 = pack4(f2u8(v0[0]), f2u8(v0[1]), f2u8(v0[2]), f2u8(v0[3]));
-    const uint32_t w1 = pack4(f2u8(v1[0]), f2u8(v1[1]), f2u8(v1[2]), f2u8(v1[3]));
-    tile[(b * 2 * SR + 2 * r) * 32 + lane] = w0;
-    tile[(b * 2 * SR + 2 * r + 1) * 32 + lane] = w1;
-    // ERGAS reference: MS(m, n), MS(m, n+1) each repeated over 2 PAN columns.
-    rep[(b * SR + r) * 32 + lane] = __byte_perm(f2u8(mn), f2u8(mn1), 0x4400u);
-    const int64_t HW = s.H * s.W;
-    const int64_t o0 = (int64_t)b * HW + (2 * m) * s.W + c.x, o1 = o0 + s.W;
-    if (alt) {
-        // Even row on the 16-byte grid (the lane at x = W-2 writes pairs),
-        // odd row 2 pixels past it: every lane takes part in the shuffles.
-        OutPtrs o{s.out_f32 ? s.out_f32 + (int64_t)b * HW : nullptr, s.out_u8 + (int64_t)b * HW};
-        if (c.active) store4(o, (2 * m) * s.W + c.x, c.two, c.two, v0);
-        store4_shifted(o, (2 * m + 1) * s.W + c.x, lane, c.active, c.two, c.last, v1);
-        return;
-    }
-    if (!c.active) return;
-    if (s.out_f32) {
-        float *p0 = s.out_f32 + o0, *p1 = s.out_f32 + o1;
-        if (a4) {
-            __stcs(reinterpret_cast<float4 *>(p0), make_float4(v0[0], v0[1], v0[2], v0[3]));
-            __stcs(reinterpret_cast<float4 *>(p1), make_float4(v1[0], v1[1], v1[2], v1[3]));
-        } else {
-            __stcs(reinterpret_cast<float2 *>(p0), make_float2(v0[0], v0[1]));
-            __stcs(reinterpret_cast<float2 *>(p1), make_float2(v1[0], v1[1]));
-            if (c.two) {
-                __stcs(reinterpret_cast<float2 *>(p0 + 2), make_float2(v0[2], v0[3]));
-                __stcs(reinterpret_cast<float2 *>(p1 + 2), make_float2(v1[2], v1[3]));
-            }
-        }
-    }
-    uint8_t *q0 = s.out_u8 + o0, *q1 = s.out_u8 + o1;
-    if (a4) {
-        __stcs(reinterpret_cast<unsigned int *>(q0), w0);
-        __stcs(reinterpret_cast<unsigned int *>(q1), w1);
-    } else {
-        __stcs(reinterpret_cast<unsigned short *>(q0), (unsigned short)(w0 & 0xffffu));
-        __stcs(reinterpret_cast<unsigned short *>(q1), (unsigned short)(w1 & 0xffffu));
-        if (c.two) {
-            __stcs(reinterpret_cast<unsigned short *>(q0 + 2), (unsigned short)(w0 >> 16));
-            __stcs(reinterpret_cast<unsigned short *>(q1 + 2), (unsigned short)(w1 >> 16));
-        }
-    }
-}
-
-// PAN rows 2m, 2m+1 of the lane into tile slot r.
-template <int NB, int SR>
-__device__ __forceinline__ void metric_pan(uint32_t *tile, int lane, int r, const float *pan0, const float *pan1) {
-    tile[(NB * 2 * SR + 2 * r) * 32 + lane] = pack4(f2u8(pan0[0]), f2u8(pan0[1]), f2u8(pan0[2]), f2u8(pan0[3]));
-    tile[(NB * 2 * SR + 2 * r + 1) * 32 + lane] = pack4(f2u8(pan1[0]), f2u8(pan1[1]), f2u8(pan1[2]), f2u8(pan1[3]));
-}
-
 template <int NB>
 struct FmLayout {
     static constexpr int K = NB + 1;                  // images: NB bands, then PAN
@@ -138,31 +80,47 @@ struct FmLayout {
     // TMEM: warps w, w + 4, w + 8, ... share a quarter of the lanes, side by side.
     static constexpr int kWarpTmem = fm_pow2_at_least(NT, 16);
     static constexpr int kTmemCols = fm_pow2_at_least((kWarps + 3) / 4 * kWarpTmem, 32);
+    static_assert(kSmem <= 227 * 1024, "shared memory of an SM");
     static_assert(NT <= 64 && kTmemCols <= 512, "TMEM columns of an SM");
 };
 
-template <int NB>
+template <int NB, int LAY>
 struct MetricEmit {
     using L = FmLayout<NB>;
     static constexpr bool kAllLanes = true;
+    static constexpr int kMode = kScalarCol;
     static constexpr int K = L::K, P = L::P, NS = L::NS, SR = L::SR;
     const SceneArgs &s;
     const LaneCols &c;
+    OutRun o;
     uint32_t *tile, *rep;
     int *gsum;
     float *qs;
     long long *se64;
     uint32_t taddr;  // this warp's TMEM cells
-    int64_t x0, m_s, m_e;
-    int lane;
-    bool a4;
-    bool alt;       // W % 4 == 2 with vector-aligned planes: even rows vectorised, odd rows shifted
+    int64_t x0;
+    int m_s, m_e, lane;
     uint32_t keep;  // bytes of this lane's 4-pixel words inside the image
     bool fresh;     // the lane's TMEM sums start over (item start, after a window row)
 
-    __device__ __forceinline__ void band(int b, int64_t m, const float *v0, const float *v1, float mn,
-                                         float mn1) const {
-        metric_band<NB, SR>(s, c, tile, rep, lane, (int)((m - m_s) & (SR - 1)), a4, alt, b, m, v0, v1, mn, mn1);
+    int r = 0;  // tile slot of the current MS row (of SR)
+
+    // Parks the band's uint8 words of PAN rows 2m, 2m+1 and its MS reference
+    // word (MS(m, n), MS(m, n+1) each repeated over 2 PAN columns) in tile
+    // slot r, and writes the fused pixels.
+    __device__ __forceinline__ void band(int b, const float *v0, const float *v1, uint32_t mn, uint32_t mn1) {
+        const uint32_t w0 = pack4u8(v0), w1 = pack4u8(v1);
+        tile[(b * 2 * SR + 2 * r) * 32 + lane] = w0;
+        tile[(b * 2 * SR + 2 * r + 1) * 32 + lane] = w1;
+        rep[(b * SR + r) * 32 + lane] = __byte_perm(mn, mn1, 0x4400u);
+        if (o.hf) {
+            store_f32<LAY>(o.f, c, lane, false, v0);
+            store_f32<LAY>(o.f + s.W, c, lane, true, v1);
+            o.f += s.out_plane;
+        }
+        store_u8<LAY>(o.u, c, lane, false, w0);
+        store_u8<LAY>(o.u + s.W, c, lane, true, w1);
+        o.u += s.out_plane;
     }
 
     // Terms of the tile's first `nr` PAN rows for the cells [LO, HI) into
@@ -261,14 +219,19 @@ struct MetricEmit {
         __syncwarp();
     }
 
-    __device__ __forceinline__ void row_end(int64_t m, const float *pan0, const float *pan1) {
-        const int r = (int)((m - m_s) & (SR - 1));
-        metric_pan<NB, SR>(tile, lane, r, pan0, pan1);
+    template <int>
+    __device__ __forceinline__ void row_end(int m, uint32_t pan0, uint32_t pan1) {
+        tile[(NB * 2 * SR + 2 * r) * 32 + lane] = pan0;
+        tile[(NB * 2 * SR + 2 * r + 1) * 32 + lane] = pan1;
+        o.next_row(2 * s.W - NB * s.out_plane);
         const bool last = m + 1 == m_e;
-        if (r != SR - 1 && !last) return;
+        if (r != SR - 1 && !last) {
+            ++r;
+            return;
+        }
         // Rows 2m' .. 2m+1 of the window row starting at PAN row y_win.
         const bool fl = (m - m_s + 1) % kFmWinMs == 0 || last;
-        const int64_t y_win = ((2 * m) / 32) * 32;
+        const int64_t y_win = ((2 * (int64_t)m) / 32) * 32;
         const bool row_full = y_win + 32 <= s.H;
         const bool win_in = row_full && x0 + 32 * ((lane >> 3) + 1) <= s.W;
         if constexpr (NB <= 6) {
@@ -284,11 +247,12 @@ struct MetricEmit {
             score_cells<B, NS, false>(2 * (r + 1), fl, win_in);
         }
         fresh = fl;
+        r = 0;
         if (fl) finish_window(row_full);
     }
 };
 
-template <typename T, int WAV, int NB>
+template <typename T, int WAV, int NB, int LAY>
 __global__ void __launch_bounds__(FmLayout<NB>::kThreads, 1)
 fuse_metrics_kernel(const __grid_constant__ SceneArgs s, double *partial, int stride, int *ctas_out,
                     int64_t strips_x, int64_t items, int R) {
@@ -322,18 +286,14 @@ fuse_metrics_kernel(const __grid_constant__ SceneArgs s, double *partial, int st
     for (int64_t it = (int64_t)warp * gridDim.x + blockIdx.x; it < items; it += nwarps) {
         const int64_t sx = it % strips_x, sy = it / strips_x;
         const int64_t x0 = sx * kWarpCols;
-        const int64_t m_s = sy * R;
-        const int64_t m_e = min(m_s + (int64_t)R, s.H >> 1);
+        const int m_s = (int)(sy * R);
+        const int m_e = (int)min((int64_t)m_s + R, s.H >> 1);
         const LaneCols c = lane_cols(x0, lane, s.W);
-        const int64_t x = x0 + 4 * lane;
+            const int64_t x = x0 + 4 * lane;
         const uint32_t keep = x + 4 <= s.W ? 0xffffffffu : (x + 2 <= s.W ? 0x0000ffffu : 0u);
-        const bool a4 = s.a4 != 0, alt = !a4 && s.alt != 0;
-        const bool lde = a4 || (alt && c.two);  // 4-pixel PAN loads on even rows
-        MetricEmit<NB> out{s, c, tile, rep, gsum, qs, se64, taddr, x0, m_s, m_e, lane, a4, alt, keep, true};
-        if (WAV == 0)
-            haar_rows<T, NB>(s, c, lde, a4, m_s, m_e, 0, NB, out);
-        else
-            d4_rows<T, NB>(s, c, lde, a4, m_s, m_e, 0, NB, out);
+        MetricEmit<NB, LAY> out{s,    c,     OutRun(s, c, 0, m_s), tile, rep, gsum, qs,
+                                se64, taddr, x0, m_s, m_e, lane, keep, true};
+        walk_rows<T, WAV, NB, LAY>(s, c, x0, m_s, m_e, 0, out);
     }
     tmem_fence_before();
     __syncthreads();
@@ -369,16 +329,18 @@ struct FmKernel {
 };
 
 template <int WAV, int NB>
-FmKernel fm_of() {
-    return {reinterpret_cast<void *>(&fuse_metrics_kernel<uint8_t, WAV, NB>), FmLayout<NB>::kThreads,
-            FmLayout<NB>::kSmem, FmLayout<NB>::kTmemCols};
+FmKernel fm_of(int lay) {
+    void *fn = lay == kVec     ? reinterpret_cast<void *>(&fuse_metrics_kernel<uint8_t, WAV, NB, kVec>)
+               : lay == kShift ? reinterpret_cast<void *>(&fuse_metrics_kernel<uint8_t, WAV, NB, kShift>)
+                               : reinterpret_cast<void *>(&fuse_metrics_kernel<uint8_t, WAV, NB, kPairs>);
+    return {fn, FmLayout<NB>::kThreads, FmLayout<NB>::kSmem, FmLayout<NB>::kTmemCols};
 }
 
-FmKernel fm_kernel(int wav, int nb) {
+FmKernel fm_kernel(int wav, int nb, int lay) {
     switch (nb) {
 #define DWTFUSE_FM(NBV) \
     case NBV:           \
-        return wav ? fm_of<1, NBV>() : fm_of<0, NBV>();
+        return wav ? fm_of<1, NBV>(lay) : fm_of<0, NBV>(lay);
         DWTFUSE_FM(1) DWTFUSE_FM(2) DWTFUSE_FM(3) DWTFUSE_FM(4) DWTFUSE_FM(5) DWTFUSE_FM(6)
         DWTFUSE_FM(7) DWTFUSE_FM(8)
 #undef DWTFUSE_FM
@@ -394,7 +356,7 @@ bool fuse_metrics_supported(const SceneArgs &s) {
 
 cudaError_t launch_fuse_metrics(const SceneArgs &s, double *pan_partial, int stride, int *ctas_dev,
                                 cudaStream_t stream) {
-    const FmKernel k = fm_kernel(s.wavelet, s.bands);
+    const FmKernel k = fm_kernel(s.wavelet, s.bands, row_layout(s.a4, s.alt));
     if (k.fn == nullptr || s.in_f32 || s.out_u8 == nullptr) return cudaErrorInvalidValue;
     int occ = 0, sms = 0;
     cudaError_t e = resident_blocks_smem(k.fn, k.threads, k.smem, &occ);

@@ -49,6 +49,7 @@ __device__ __forceinline__ void bulk_wait_read() {
 template <int NB>
 struct StagedEmit {
     static constexpr bool kAllLanes = true;  // every lane reaches the row barrier
+    static constexpr int kMode = 0;
     const SceneArgs &s;
     const LaneCols &c;
     float *buf;    // two slots of [NB][2][kStCols] floats
@@ -56,24 +57,26 @@ struct StagedEmit {
     int ncols;     // columns of the strip inside the image (a multiple of 4)
     int b0;        // first band of the launch's chunk
     int *rowc;     // the CTA's row count: row k fills slot k & 1
+    bool hu;       // uint8 output wanted
+    uint8_t *u;    // its band b0, the current MS row's first image row, column x
 
     __device__ __forceinline__ float *slot() const { return buf + (*rowc & 1) * (NB * 2 * kStCols); }
 
-    __device__ __forceinline__ void band(int b, int64_t m, const float *v0, const float *v1, float, float) const {
+    template <typename M>
+    __device__ __forceinline__ void band(int b, const float *v0, const float *v1, M, M) {
+        u += b ? s.out_plane : 0;
         if (!c.active) return;
-        const int col = c.x - (int)X0;
-        float *row = slot() + b * 2 * kStCols + col;
+        float *row = slot() + b * 2 * kStCols + (c.x - (int)X0);
         *reinterpret_cast<float4 *>(row) = make_float4(v0[0], v0[1], v0[2], v0[3]);
         *reinterpret_cast<float4 *>(row + kStCols) = make_float4(v1[0], v1[1], v1[2], v1[3]);
-        if (s.out_u8) {
-            const int64_t W = s.W, y = 2 * (m - s.m_lo);
-            OutPtrs o{nullptr, s.out_u8 + (int64_t)(b0 + b) * s.out_plane};
-            store4(o, y * W + c.x, true, c.two, v0);
-            store4(o, (y + 1) * W + c.x, true, c.two, v1);
+        if (hu) {
+            store_u8<kVec>(u, c, 0, false, pack4u8(v0));
+            store_u8<kVec>(u + s.W, c, 0, true, pack4u8(v1));
         }
     }
 
-    __device__ __forceinline__ void row_end(int64_t m, const float *, const float *) const {
+    template <int>
+    __device__ __forceinline__ void row_end(int m, uint32_t, uint32_t) {
         // Make this thread's shared-memory writes visible to the bulk copy engine.
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         const int t = threadIdx.x;
@@ -81,13 +84,14 @@ struct StagedEmit {
         __syncthreads();
         if (t < 2 * NB) {
             const int b = t >> 1, r = t & 1;
-            const int64_t y = 2 * (m - s.m_lo) + r;
+            const int64_t y = 2 * (int64_t)(m - s.m_lo) + r;
             float *dst = s.out_f32 + (int64_t)(b0 + b) * s.out_plane + y * s.W + X0;
             asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(dst),
                          "r"(st_smem(slot() + (b * 2 + r) * kStCols)), "r"((unsigned)ncols * 4u)
                          : "memory");
             asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
         }
+        u += 2 * s.W - (NB - 1) * s.out_plane;
         ++*rowc;
     }
 };
@@ -95,16 +99,15 @@ struct StagedEmit {
 // One CTA item: columns [X0, X0 + 1024), MS rows [m_s, m_e), bands
 // [b0, b0 + NB).  Every thread of the CTA calls it, with the same row count.
 template <typename T, int WAV, int NB>
-__device__ __forceinline__ void staged_item(const SceneArgs &s, float *buf, int64_t X0, int64_t m_s, int64_t m_e,
-                                            int b0, int *rowc) {
+__device__ __forceinline__ void staged_item(const SceneArgs &s, float *buf, int64_t X0, int m_s, int m_e, int b0,
+                                            int *rowc) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const LaneCols c = lane_cols(X0 + (int64_t)warp * kWarpCols, lane, s.W);  // warps past W: idle lanes
+    const int64_t x0 = X0 + (int64_t)warp * kWarpCols;
+    const LaneCols c = lane_cols(x0, lane, s.W);  // warps past W: idle lanes
     const int ncols = (int)min((int64_t)kStCols, s.W - X0);
-    StagedEmit<NB> out{s, c, buf, X0, ncols, b0, rowc};
-    if (WAV == 0)
-        haar_rows<T, NB>(s, c, true, true, m_s, m_e, b0, NB, out);
-    else
-        d4_rows<T, NB>(s, c, true, true, m_s, m_e, b0, NB, out);
+    uint8_t *u = s.out_u8 + (int64_t)b0 * s.out_plane + (int64_t)(2 * (m_s - s.m_lo)) * s.W + c.x;
+    StagedEmit<NB> out{s, c, buf, X0, ncols, b0, rowc, s.out_u8 != nullptr, u};
+    walk_rows<T, WAV, NB, kVec>(s, c, x0, m_s, m_e, b0, out);
 }
 
 __device__ __forceinline__ void bulk_drain() {
@@ -121,8 +124,8 @@ fuse_staged_kernel(const __grid_constant__ SceneArgs s, int b0, int64_t strips_c
     int rowc = 0;
     for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
         const int64_t sx = it % strips_cta, sy = it / strips_cta;
-        const int64_t m_s = s.m_lo + sy * R;
-        staged_item<T, WAV, NB>(s, st_buf, sx * kStCols, m_s, min(m_s + (int64_t)R, (int64_t)s.m_hi), b0, &rowc);
+        const int m_s = s.m_lo + (int)(sy * R);
+        staged_item<T, WAV, NB>(s, st_buf, sx * kStCols, m_s, min(m_s + R, s.m_hi), b0, &rowc);
     }
     bulk_drain();
 }

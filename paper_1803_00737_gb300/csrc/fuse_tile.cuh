@@ -19,6 +19,18 @@
 // (periodic wrap at the image edges, Eq. 5-6 and 13-14), and a vertical
 // pipeline keeps the row-synthesised values of MS row m-1 for row m.  Loads
 // use the read-only path; fused rows are written with streaming stores.
+//
+// What bounds the walkers: with a float output HBM writes; with only the uint8
+// product, or scoring it, the instructions per pixel and the latency of a
+// step's loads (16 warps per SM).  So: paired FP32, byte conversions on the
+// fast pipes, running addresses instead of 64-bit products per band, row
+// layouts and inner strips (no wrapped columns) as template instances.  Per
+// warp step of 8 bands 1000 -> 585 instructions; against the walkers with
+// run-time layouts and scalar FP32: 7480 x 8140 x 8 to uint8 279 -> 185 us,
+// scored 9414^2 x 8 1022 -> 894 us and 16384^2 x 6 1624 -> 1589 us a pass.
+// Streaming the rows through a per-warp cp.async ring instead of registers
+// (615 instructions per step) was slower: 7480 x 8140 x 8 237 us, 16384^2 x 6
+// scored 1831 us.
 #pragma once
 
 #include <cstdint>
@@ -119,41 +131,6 @@ __device__ __forceinline__ void store4(const OutPtrs &o, int64_t off, bool a4, b
     }
 }
 
-// Writes the 4 fused pixels (y, x..x+3) of one band on a row whose start is 2
-// pixels past a 16-byte boundary (W = 2 mod 4, odd rows): every lane but the
-// first writes the aligned vector (y, x-2..x+1), taking pixels x-2, x-1 from
-// its left neighbour; lane 0 writes (x, x+1) and the last lane of the strip
-// (x + 4 >= W or lane 31) also writes (x+2, x+3).  Every lane of the warp must
-// call it (warp shuffles); `active` masks the stores.
-__device__ __forceinline__ void store4_shifted(const OutPtrs &o, int64_t off, int lane, bool active,
-                                               bool two, bool last, const float *v) {
-    if (o.f32) {
-        const float p2 = __shfl_up_sync(0xffffffffu, v[2], 1);
-        const float p3 = __shfl_up_sync(0xffffffffu, v[3], 1);
-        if (active) {
-            float *p = o.f32 + off;
-            if (lane > 0)
-                __stcs(reinterpret_cast<float4 *>(p - 2), make_float4(p2, p3, v[0], v[1]));
-            else
-                __stcs(reinterpret_cast<float2 *>(p), make_float2(v[0], v[1]));
-            if (two && last) __stcs(reinterpret_cast<float2 *>(p + 2), make_float2(v[2], v[3]));
-        }
-    }
-    if (o.u8) {
-        const uint32_t q0 = f2u8(v[0]), q1 = f2u8(v[1]), q2 = f2u8(v[2]), q3 = f2u8(v[3]);
-        const uint32_t w = pack4(q0, q1, q2, q3);
-        const uint32_t pw = __shfl_up_sync(0xffffffffu, w, 1);
-        if (active) {
-            uint8_t *p = o.u8 + off;
-            if (lane > 0)
-                __stcs(reinterpret_cast<unsigned int *>(p - 2), __byte_perm(pw, w, 0x5432u));
-            else
-                __stcs(reinterpret_cast<unsigned short *>(p), (unsigned short)(w & 0xffffu));
-            if (two && last) __stcs(reinterpret_cast<unsigned short *>(p + 2), (unsigned short)(w >> 16));
-        }
-    }
-}
-
 // ------------------------------------------------------------------ scene
 
 // Everything a warp needs about one scene.  Band pointers are typed by the
@@ -240,120 +217,424 @@ __device__ __forceinline__ void d4_rowpass(const float *v, float *r) {
     r[2] = fmaf(kH3, v[7], fmaf(kH2, v[6], fmaf(kH1, v[5], kH0 * v[4])));
 }
 
+// ------------------------------------------------------------------ row layouts
+//
+// kVec:   W % 4 == 0 and every image row starts on a 4-pixel boundary.
+// kShift: W % 4 == 2 with aligned planes: even rows start on a 4-pixel
+//         boundary, odd rows 2 pixels past one.
+// kPairs: anything else (every access is a pixel pair).
+enum : int { kPairs = 0, kVec = 1, kShift = 2 };
+
+__device__ __host__ inline int row_layout(int32_t a4, int32_t alt) { return a4 ? kVec : (alt ? kShift : kPairs); }
+
+// A strip is inner when no lane's taps (columns x-2 .. x+5, MS columns
+// n-1 .. n+1) leave the image row: the wrapped columns are then plain offsets
+// and every lane is active.  The same for the whole warp.
+__device__ __forceinline__ bool strip_inner(int64_t x0, int64_t W) { return x0 > 0 && x0 + kWarpCols + 2 <= W; }
+
+// ------------------------------------------------------------------ paired FP32
+//
+// Two FP32 operations per instruction (fma / mul / add .f32x2, each lane
+// rounded as the scalar operation): the same arithmetic pipe time, half the
+// issue slots.  The forward walkers were issue-bound (uint8 output, 8 bands:
+// 74 % of issue slots, about 1000 instructions per warp and MS row).
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pk2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void up2(f32x2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// 4 floats -> 4 uint8 (clamped, rounded half to even; NaN -> 0) in one word.
+// cvt.rni.s32 saturates, and cvt.pack clamps two values to bytes at once: 6
+// instructions against 4 saturating conversions and 3 byte permutes.
+__device__ __forceinline__ uint32_t pack4u8(const float *v) {
+    int i0, i1, i2, i3;
+    asm("cvt.rni.s32.f32 %0, %1;" : "=r"(i0) : "f"(v[0]));
+    asm("cvt.rni.s32.f32 %0, %1;" : "=r"(i1) : "f"(v[1]));
+    asm("cvt.rni.s32.f32 %0, %1;" : "=r"(i2) : "f"(v[2]));
+    asm("cvt.rni.s32.f32 %0, %1;" : "=r"(i3) : "f"(v[3]));
+    uint32_t hi, w;
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, 0;" : "=r"(hi) : "r"(i3), "r"(i2));
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(w) : "r"(i1), "r"(i0), "r"(hi));
+    return w;
+}
+
+// ------------------------------------------------------------------ raw loads
+//
+// A walker's inputs as loaded: uint8 words and bytes (a third of the floats'
+// registers), converted where they are used.
+
+template <typename T>
+struct RawRow;  // PAN columns x-2 .. x+5 of one image row
+template <>
+struct RawRow<uint8_t> {
+    uint32_t a, b, c, d;
+};
+template <>
+struct RawRow<float> {
+    float v[8];
+};
+
+// W8: all 8 columns (D4); else columns x .. x+3 only (Haar).  SHIFT: the row
+// starts 2 pixels past a 4-pixel boundary (kShift, odd rows).
+template <int LAY, bool INNER, bool SHIFT, bool W8>
+__device__ __forceinline__ void load_raw(const uint8_t *row, const LaneCols &c, RawRow<uint8_t> &r) {
+    if (LAY == kVec) {
+        r.b = __ldg(reinterpret_cast<const unsigned int *>(row + c.x));
+        if (W8) {
+            if (INNER) {
+                r.a = __ldg(reinterpret_cast<const unsigned short *>(row + c.x - 2));
+                r.c = __ldg(reinterpret_cast<const unsigned short *>(row + c.x + 4));
+            } else {
+                r.a = __ldg(reinterpret_cast<const unsigned short *>(row + c.cm));
+                r.c = __ldg(reinterpret_cast<const unsigned short *>(row + c.c4));
+            }
+        }
+        return;
+    }
+    if (LAY == kShift && INNER) {
+        const uint8_t *p = row + c.x;
+        if (SHIFT) {
+            if (W8) {
+                r.a = __ldg(reinterpret_cast<const unsigned int *>(p - 2));
+                r.b = __ldg(reinterpret_cast<const unsigned int *>(p + 2));
+            } else {
+                r.a = __ldg(reinterpret_cast<const unsigned short *>(p));
+                r.b = __ldg(reinterpret_cast<const unsigned short *>(p + 2));
+            }
+        } else {
+            r.b = __ldg(reinterpret_cast<const unsigned int *>(p));
+            if (W8) {
+                r.a = __ldg(reinterpret_cast<const unsigned short *>(p - 2));
+                r.c = __ldg(reinterpret_cast<const unsigned short *>(p + 4));
+            }
+        }
+        return;
+    }
+    if (W8) {
+        r.a = __ldg(reinterpret_cast<const unsigned short *>(row + c.cm));
+        r.d = __ldg(reinterpret_cast<const unsigned short *>(row + c.c4));
+    }
+    r.b = __ldg(reinterpret_cast<const unsigned short *>(row + c.x));
+    r.c = __ldg(reinterpret_cast<const unsigned short *>(row + c.c2));
+}
+
+template <int LAY, bool INNER, bool SHIFT, bool W8>
+__device__ __forceinline__ void load_raw(const float *row, const LaneCols &c, RawRow<float> &r) {
+    if (LAY == kVec || (LAY == kShift && INNER)) {
+        const float *p = row + c.x;
+        if (LAY == kShift && SHIFT) {
+            if (W8) {
+                ld4(p - 2, r.v);
+                ld4(p + 2, r.v + 4);
+            } else {
+                ld2(p, r.v[2], r.v[3]);
+                ld2(p + 2, r.v[4], r.v[5]);
+            }
+            return;
+        }
+        ld4(p, r.v + 2);
+        if (W8) {
+            if (LAY == kShift || INNER) {
+                ld2(p - 2, r.v[0], r.v[1]);
+                ld2(p + 4, r.v[6], r.v[7]);
+            } else {
+                ld2(row + c.cm, r.v[0], r.v[1]);
+                ld2(row + c.c4, r.v[6], r.v[7]);
+            }
+        }
+        return;
+    }
+    ld2(row + c.x, r.v[2], r.v[3]);
+    ld2(row + c.c2, r.v[4], r.v[5]);
+    if (W8) {
+        ld2(row + c.cm, r.v[0], r.v[1]);
+        ld2(row + c.c4, r.v[6], r.v[7]);
+    }
+}
+
+// The row's words: lo = columns x-2 .. x+1, hi = x+2 .. x+5 (Haar: only the
+// own columns x .. x+3, in lo).
+template <int LAY, bool INNER, bool SHIFT, bool W8>
+__device__ __forceinline__ void raw_words(const RawRow<uint8_t> &r, uint32_t &lo, uint32_t &hi) {
+    if (LAY == kVec || (LAY == kShift && INNER && !SHIFT)) {
+        if (W8) {
+            lo = __byte_perm(r.a, r.b, 0x5410u);
+            hi = __byte_perm(r.b, r.c, 0x5432u);
+        } else {
+            lo = r.b;
+        }
+    } else if (LAY == kShift && INNER) {
+        if (W8) {
+            lo = r.a;
+            hi = r.b;
+        } else {
+            lo = __byte_perm(r.a, r.b, 0x5410u);
+        }
+    } else if (W8) {
+        lo = __byte_perm(r.a, r.b, 0x5410u);
+        hi = __byte_perm(r.c, r.d, 0x5410u);
+    } else {
+        lo = __byte_perm(r.b, r.c, 0x5410u);
+    }
+}
+
+// Columns x-2 .. x+5 (D4: v[0..7]; Haar: only v[2..5]) as floats, and the own
+// columns' word x .. x+3 (uint8 only).
+template <int LAY, bool INNER, bool SHIFT, bool W8>
+__device__ __forceinline__ void raw_floats(const RawRow<uint8_t> &r, float *v, uint32_t &own) {
+    uint32_t lo, hi = 0;
+    raw_words<LAY, INNER, SHIFT, W8>(r, lo, hi);
+    if (W8) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k] = byte_f(lo, k);
+            v[4 + k] = byte_f(hi, k);
+        }
+        own = __byte_perm(lo, hi, 0x5432u);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[2 + k] = byte_f(lo, k);
+        own = lo;
+    }
+}
+template <int LAY, bool INNER, bool SHIFT, bool W8>
+__device__ __forceinline__ void raw_floats(const RawRow<float> &r, float *v, uint32_t &own) {
+#pragma unroll
+    for (int k = W8 ? 0 : 2; k < (W8 ? 8 : 6); ++k) v[k] = r.v[k];
+    own = 0;
+}
+
+// One MS value, raw and as a float.  uint8: the byte in a 32-bit register
+// (cvt.rn.f32.u32 runs at 64 lanes a clock and SM, cvt.rn.f32.u8 at 16).
+template <typename T>
+struct RawMs;
+template <>
+struct RawMs<uint8_t> {
+    typedef uint32_t type;
+};
+template <>
+struct RawMs<float> {
+    typedef float type;
+};
+__device__ __forceinline__ uint32_t ld_ms(const uint8_t *p) {
+    uint32_t r;
+    asm("ld.global.nc.u8 %0, [%1];" : "=r"(r) : "l"(p));
+    return r;
+}
+__device__ __forceinline__ float ld_ms(const float *p) { return __ldg(p); }
+__device__ __forceinline__ float ms_f(uint32_t v) {
+    float f;
+    asm("cvt.rn.f32.u32 %0, %1;" : "=f"(f) : "r"(v));
+    return f;
+}
+__device__ __forceinline__ float ms_f(float v) { return v; }
+
 // ------------------------------------------------------------------ row walkers
 //
 // A walker takes one lane's columns (LaneCols) down MS rows [m_s, m_e) and
 // hands every band's two fused PAN rows 2m, 2m+1 (4 pixels per lane) to an
-// emitter: out.band(b, m, v0, v1, mn, mn1) per band, with the band's MS values
-// at MS columns n = x/2 and n+1 (the ones the lane's pixels were made from),
-// then out.row_end(m, pan0, pan1) once per MS row with the lane's PAN pixels
-// of rows 2m and 2m+1.  Emit::kAllLanes: the emitter needs every lane (warp
-// shuffles), so idle lanes compute on column 0 and call it too.  ld_even /
-// ld_odd select the 4-pixel PAN loads on even / odd rows.
+// emitter: out.band(b, v0, v1, mn, mn1) per band, with the band's raw MS
+// values at MS columns n = x/2 and n+1 (the ones the lane's pixels were made
+// from), then out.row_end(m, own0, own1) once per MS row with the lane's PAN
+// words of rows 2m and 2m+1 (uint8 images).  Emit::kAllLanes: the emitter
+// needs every lane (warp shuffles, barriers), so idle lanes compute on column
+// 0 and call it too.  Addresses run: one PAN pointer and one MS offset are
+// advanced per MS row.
+
+// Emit::kMode, a sum of:
+//   kAheadPan, kAheadMs  load the next MS row's PAN rows / MS values one row
+//                        ahead (raw words and bytes; they stay in registers
+//                        for a whole row)
+//   kScalarCol           column synthesis in scalar FP32 (its constants are
+//                        immediates; the paired form holds 8 registers of
+//                        them, which spill in the scoring kernel)
+// Measured per kernel (see there): ahead pays where few bands leave registers
+// free, and costs where the walker then spills.
+enum : int { kAheadPan = 1, kAheadMs = 2, kScalarCol = 4 };
 
 // Haar (Eq. 1-2, 11-12).
-template <typename T, int NB, class Emit>
-__device__ __forceinline__ void haar_rows(const SceneArgs &s, const LaneCols &c, bool ld_even, bool ld_odd,
-                                          int64_t m_s, int64_t m_e, int b0, int nb, Emit &out) {
+template <typename T, int NB, int LAY, bool INNER, class Emit>
+__device__ __forceinline__ void haar_rows(const SceneArgs &s, const LaneCols &c, int m_s, int m_e,
+                                          int b0, Emit &out) {
+    typedef typename RawMs<T>::type M;
+    constexpr bool kPanA = (Emit::kMode & kAheadPan) != 0, kMsA = (Emit::kMode & kAheadMs) != 0;
     const int64_t W = s.W, W2 = W >> 1;
-    const T *pan = static_cast<const T *>(s.pan);
-    for (int64_t m = m_s; m < m_e; ++m) {
-        float p0[4], p1[4];
-        load_row4(pan + (2 * m) * W, c, ld_even, p0);
-        load_row4(pan + (2 * m + 1) * W, c, ld_odd, p1);
-        float mv[NB][2];
+    const T *pan = static_cast<const T *>(s.pan) + (int64_t)(2 * m_s) * W;
+    int64_t mo = (int64_t)m_s * W2 + c.nB;
+    const int dC = c.nC - c.nB;
+    RawRow<T> ra, rb;
+    M mr[NB][2];
+    auto load_pan = [&]() {
+        load_raw<LAY, INNER, false, false>(pan, c, ra);
+        load_raw<LAY, INNER, true, false>(pan + W, c, rb);
+        pan += 2 * W;
+    };
+    auto load_ms = [&](int b) {
+        const T *ms = static_cast<const T *>(s.ms[b0 + b]) + mo;
+        mr[b][0] = ld_ms(ms);
+        mr[b][1] = INNER ? ld_ms(ms + 1) : ld_ms(ms + dC);
+    };
+    if (kPanA) load_pan();
+    if (kMsA) {
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            if (b < nb) {
-                const T *ms = static_cast<const T *>(s.ms[b0 + b]) + m * W2;
-                mv[b][0] = ld1(ms + c.nB);
-                mv[b][1] = ld1(ms + c.nC);
-            }
+        for (int b = 0; b < NB; ++b) load_ms(b);
+    }
+#pragma unroll 1
+    for (int m = m_s; m < m_e; ++m) {
+        const bool more = m + 1 < m_e;
+        if (!kPanA) load_pan();
+        if (!kMsA) {
+#pragma unroll
+            for (int b = 0; b < NB; ++b) load_ms(b);
         }
-        if (!Emit::kAllLanes && !c.active) continue;
+        mo += W2;
+        float p0[8], p1[8];
+        uint32_t own0, own1;
+        raw_floats<LAY, INNER, false, false>(ra, p0, own0);
+        raw_floats<LAY, INNER, true, false>(rb, p1, own1);
+        if (kPanA && more) load_pan();
         // Eq. 1 along the rows, then along the columns: LL = 2x2 mean (exact in FP32 for 8-bit input).
-        const float ll0 = ((p0[0] + p0[1]) * 0.5f + (p1[0] + p1[1]) * 0.5f) * 0.5f;
-        const float ll1 = ((p0[2] + p0[3]) * 0.5f + (p1[2] + p1[3]) * 0.5f) * 0.5f;
+        const float ll0 = ((p0[2] + p0[3]) * 0.5f + (p1[2] + p1[3]) * 0.5f) * 0.5f;
+        const float ll1 = ((p0[4] + p0[5]) * 0.5f + (p1[4] + p1[5]) * 0.5f) * 0.5f;
+        const f32x2 pa0 = pk2(p0[2], p0[3]), pa1 = pk2(p0[4], p0[5]);
+        const f32x2 pb0 = pk2(p1[2], p1[3]), pb1 = pk2(p1[4], p1[5]);
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
-            if (b < nb) {
-                // Eq. 11-12 on an LL-only image repeat each coefficient over its 2x2 block.
-                const float e0 = fmaf(s.gain, mv[b][0], -ll0);
-                const float e1 = fmaf(s.gain, mv[b][1], -ll1);
-                float v[4] = {p0[0] + e0, p0[1] + e0, p0[2] + e1, p0[3] + e1};
-                float w[4] = {p1[0] + e0, p1[1] + e0, p1[2] + e1, p1[3] + e1};
-                out.band(b, m, v, w, mv[b][0], mv[b][1]);
-            }
+            // Eq. 11-12 on an LL-only image repeat each coefficient over its 2x2 block.
+            const M m0 = mr[b][0], m1 = mr[b][1];
+            if (kMsA && more) load_ms(b);  // the next row's, once this row's are taken
+            const float e0 = fmaf(s.gain, ms_f(m0), -ll0);
+            const float e1 = fmaf(s.gain, ms_f(m1), -ll1);
+            const f32x2 ee0 = pk2(e0, e0), ee1 = pk2(e1, e1);
+            float v[4], w[4];
+            up2(add2(pa0, ee0), v[0], v[1]);
+            up2(add2(pa1, ee1), v[2], v[3]);
+            up2(add2(pb0, ee0), w[0], w[1]);
+            up2(add2(pb1, ee1), w[2], w[3]);
+            out.band(b, v, w, m0, m1);
         }
-        out.row_end(m, p0, p1);
+        out.template row_end<NB>(m, own0, own1);
     }
 }
 
 // D4 (Eq. 3-10, 13-16).
-template <typename T, int NB, class Emit>
-__device__ __forceinline__ void d4_rows(const SceneArgs &s, const LaneCols &c, bool ld_even, bool ld_odd,
-                                        int64_t m_s, int64_t m_e, int b0, int nb, Emit &out) {
-    const int64_t W = s.W, H = s.H, W2 = W >> 1, H2 = H >> 1;
-    const T *pan = static_cast<const T *>(s.pan);
+template <typename T, int NB, int LAY, bool INNER, class Emit>
+__device__ __forceinline__ void d4_rows(const SceneArgs &s, const LaneCols &c, int m_s, int m_e, int b0,
+                                        Emit &out) {
+    typedef typename RawMs<T>::type M;
+    constexpr bool kPanA = (Emit::kMode & kAheadPan) != 0, kMsA = (Emit::kMode & kAheadMs) != 0;
+    const int64_t W = s.W, H = s.H, W2 = W >> 1;
+    const int H2 = (int)(H >> 1);
+    const T *const img = static_cast<const T *>(s.pan);
     const float gain = s.gain;
+    const f32x2 h01 = pk2(kH0, kH1), h23 = pk2(kH2, kH3);
+    const f32x2 h00 = pk2(kH0, kH0), h11 = pk2(kH1, kH1), h22 = pk2(kH2, kH2), h33 = pk2(kH3, kH3);
+    const int dA = c.nA - c.nB, dC = c.nC - c.nB;
+
+    // Row synthesis (Eq. 15-16 on an LL-only row, wrap of Eq. 13-14 via nA) of
+    // E_b at PAN columns x .. x+3, as the pairs (x, x+1) and (x+2, x+3).
+    auto synth = [&](const M *mv, const float *ll, f32x2 &lo, f32x2 &hi) {
+        const float eA = fmaf(gain, ms_f(mv[0]), -ll[0]);
+        const float eB = fmaf(gain, ms_f(mv[1]), -ll[1]);
+        const float eC = fmaf(gain, ms_f(mv[2]), -ll[2]);
+        const f32x2 bb = pk2(eB, eB);
+        lo = fma2(h23, pk2(eA, eA), mul2(h01, bb));
+        hi = fma2(h23, bb, mul2(h01, pk2(eC, eC)));
+    };
+    M mr[NB][3];
+    auto load_ms = [&](int b, int64_t mo) {
+        const T *ms = static_cast<const T *>(s.ms[b0 + b]) + mo;
+        mr[b][0] = INNER ? ld_ms(ms - 1) : ld_ms(ms + dA);
+        mr[b][1] = ld_ms(ms);
+        mr[b][2] = INNER ? ld_ms(ms + 1) : ld_ms(ms + dC);
+    };
 
     // Prologue: MS row mp = m_s - 1 (periodic) needs PAN rows 2mp .. 2mp+3.
-    const int64_t mp = wrap(m_s - 1, H2);
+    const int mp = m_s > 0 ? m_s - 1 : H2 - 1;
     float r0[3], r1[3], r2[3], r3[3];
-    float pc[4], pd[4];  // own PAN pixels of rows 2m, 2m+1 for the current m
+    f32x2 pc[2], pd[2];  // own PAN pixels of rows 2m, 2m+1 for the current m
+    uint32_t own0, own1;
+    f32x2 hprev[NB][2];  // row synthesis of E_b(m-1, .) at PAN columns x .. x+3
+    RawRow<T> ra, rb;
     {
+        RawRow<T> q0, q1;
+        const T *p = img + (int64_t)(2 * mp) * W;
+        load_raw<LAY, INNER, false, true>(p, c, q0);
+        load_raw<LAY, INNER, true, true>(p + W, c, q1);
+        p = img + (int64_t)(2 * m_s) * W;
+        load_raw<LAY, INNER, false, true>(p, c, ra);
+        load_raw<LAY, INNER, true, true>(p + W, c, rb);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) load_ms(b, (int64_t)mp * W2 + c.nB);
         float v[8];
-        load_row8(pan + (2 * mp) * W, c, ld_even, v);
+        raw_floats<LAY, INNER, false, true>(q0, v, own0);
         d4_rowpass(v, r0);
-        load_row8(pan + (2 * mp + 1) * W, c, ld_odd, v);
+        raw_floats<LAY, INNER, true, true>(q1, v, own0);
         d4_rowpass(v, r1);
-        load_row8(pan + wrap(2 * mp + 2, H) * W, c, ld_even, v);
+        raw_floats<LAY, INNER, false, true>(ra, v, own0);
         d4_rowpass(v, r2);
-        pc[0] = v[2]; pc[1] = v[3]; pc[2] = v[4]; pc[3] = v[5];
-        load_row8(pan + wrap(2 * mp + 3, H) * W, c, ld_odd, v);
+        pc[0] = pk2(v[2], v[3]);
+        pc[1] = pk2(v[4], v[5]);
+        raw_floats<LAY, INNER, true, true>(rb, v, own1);
         d4_rowpass(v, r3);
-        pd[0] = v[2]; pd[1] = v[3]; pd[2] = v[4]; pd[3] = v[5];
-    }
-    // hprev[b][q]: row synthesis of E_b(m-1, .) at PAN column x+q.
-    float hprev[NB][4];
-    {
+        pd[0] = pk2(v[2], v[3]);
+        pd[1] = pk2(v[4], v[5]);
         float ll[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k)
             ll[k] = fmaf(kH3, r3[k], fmaf(kH2, r2[k], fmaf(kH1, r1[k], kH0 * r0[k])));
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            if (b < nb) {
-                const T *ms = static_cast<const T *>(s.ms[b0 + b]) + mp * W2;
-                const float eA = fmaf(gain, ld1(ms + c.nA), -ll[0]);
-                const float eB = fmaf(gain, ld1(ms + c.nB), -ll[1]);
-                const float eC = fmaf(gain, ld1(ms + c.nC), -ll[2]);
-                hprev[b][0] = fmaf(kH2, eA, kH0 * eB);
-                hprev[b][1] = fmaf(kH3, eA, kH1 * eB);
-                hprev[b][2] = fmaf(kH2, eB, kH0 * eC);
-                hprev[b][3] = fmaf(kH3, eB, kH1 * eC);
-            }
-        }
+        for (int b = 0; b < NB; ++b) synth(mr[b], ll, hprev[b][0], hprev[b][1]);
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) { r0[k] = r2[k]; r1[k] = r3[k]; }
 
-    for (int64_t m = m_s; m < m_e; ++m) {
-        // Loads first (PAN rows 2m+2, 2m+3 and every band's MS row m), so their
-        // latencies overlap.
-        float va[8], vb[8];
-        load_row8(pan + wrap(2 * m + 2, H) * W, c, ld_even, va);
-        load_row8(pan + wrap(2 * m + 3, H) * W, c, ld_odd, vb);
-        float mv[NB][3];
+    // PAN rows 2m+2, 2m+3 (periodic: past the last row comes row 0).
+    const T *pan = img + (int64_t)(m_s + 1 < H2 ? 2 * m_s + 2 : 0) * W;
+    int64_t mo = (int64_t)m_s * W2 + c.nB;
+    auto load_pan = [&](int m) {  // the PAN rows MS row m adds
+        load_raw<LAY, INNER, false, true>(pan, c, ra);
+        load_raw<LAY, INNER, true, true>(pan + W, c, rb);
+        pan = m + 2 == H2 ? img : pan + 2 * W;
+    };
+    if (kPanA) load_pan(m_s);
+    if (kMsA) {
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            if (b < nb) {
-                const T *ms = static_cast<const T *>(s.ms[b0 + b]) + m * W2;
-                mv[b][0] = ld1(ms + c.nA);
-                mv[b][1] = ld1(ms + c.nB);
-                mv[b][2] = ld1(ms + c.nC);
-            }
+        for (int b = 0; b < NB; ++b) load_ms(b, mo);
+    }
+#pragma unroll 1
+    for (int m = m_s; m < m_e; ++m) {
+        const bool more = m + 1 < m_e;
+        if (!kPanA) load_pan(m);
+        if (!kMsA) {
+#pragma unroll
+            for (int b = 0; b < NB; ++b) load_ms(b, mo);
         }
+        mo += W2;
+        float va[8], vb[8];
+        uint32_t nown0, nown1;
+        raw_floats<LAY, INNER, false, true>(ra, va, nown0);
+        raw_floats<LAY, INNER, true, true>(rb, vb, nown1);
+        if (kPanA && more) load_pan(m + 1);
         d4_rowpass(va, r2);
         d4_rowpass(vb, r3);
         float ll[3];
@@ -362,83 +643,175 @@ __device__ __forceinline__ void d4_rows(const SceneArgs &s, const LaneCols &c, b
             ll[k] = fmaf(kH3, r3[k], fmaf(kH2, r2[k], fmaf(kH1, r1[k], kH0 * r0[k])));
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
-            if (b < nb) {
-                const float eA = fmaf(gain, mv[b][0], -ll[0]);
-                const float eB = fmaf(gain, mv[b][1], -ll[1]);
-                const float eC = fmaf(gain, mv[b][2], -ll[2]);
-                // Row synthesis (Eq. 15-16 on an LL-only row, wrap of Eq. 13-14 via nA).
-                float hc[4];
-                hc[0] = fmaf(kH2, eA, kH0 * eB);
-                hc[1] = fmaf(kH3, eA, kH1 * eB);
-                hc[2] = fmaf(kH2, eB, kH0 * eC);
-                hc[3] = fmaf(kH3, eB, kH1 * eC);
-                // Column synthesis: row 2m takes h0 (row m) and h2 (row m-1), row 2m+1 takes h1 and h3.
-                float v0[4], v1[4];
+            const M mv[3] = {mr[b][0], mr[b][1], mr[b][2]};
+            if (kMsA && more) load_ms(b, mo);  // the next row's, once this row's are taken
+            f32x2 hc[2];
+            synth(mv, ll, hc[0], hc[1]);
+            // Column synthesis: row 2m takes h0 (row m) and h2 (row m-1), row 2m+1 takes h1 and h3.
+            float v0[4], v1[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    v0[q] = fmaf(kH2, hprev[b][q], fmaf(kH0, hc[q], pc[q]));
-                    v1[q] = fmaf(kH3, hprev[b][q], fmaf(kH1, hc[q], pd[q]));
-                    hprev[b][q] = hc[q];
+            for (int q = 0; q < 2; ++q) {
+                if constexpr ((Emit::kMode & kScalarCol) != 0) {
+                    float g0, g1, x0, x1, c0, c1, d0, d1;
+                    up2(hprev[b][q], g0, g1);
+                    up2(hc[q], x0, x1);
+                    up2(pc[q], c0, c1);
+                    up2(pd[q], d0, d1);
+                    v0[2 * q] = fmaf(kH2, g0, fmaf(kH0, x0, c0));
+                    v0[2 * q + 1] = fmaf(kH2, g1, fmaf(kH0, x1, c1));
+                    v1[2 * q] = fmaf(kH3, g0, fmaf(kH1, x0, d0));
+                    v1[2 * q + 1] = fmaf(kH3, g1, fmaf(kH1, x1, d1));
+                } else {
+                    up2(fma2(h22, hprev[b][q], fma2(h00, hc[q], pc[q])), v0[2 * q], v0[2 * q + 1]);
+                    up2(fma2(h33, hprev[b][q], fma2(h11, hc[q], pd[q])), v1[2 * q], v1[2 * q + 1]);
                 }
-                out.band(b, m, v0, v1, mv[b][1], mv[b][2]);
+                hprev[b][q] = hc[q];
             }
+            out.band(b, v0, v1, mv[1], mv[2]);
         }
-        out.row_end(m, pc, pd);
+        out.template row_end<NB>(m, own0, own1);
 #pragma unroll
         for (int k = 0; k < 3; ++k) { r0[k] = r2[k]; r1[k] = r3[k]; }
-        pc[0] = va[2]; pc[1] = va[3]; pc[2] = va[4]; pc[3] = va[5];
-        pd[0] = vb[2]; pd[1] = vb[3]; pd[2] = vb[4]; pd[3] = vb[5];
+        pc[0] = pk2(va[2], va[3]);
+        pc[1] = pk2(va[4], va[5]);
+        pd[0] = pk2(vb[2], vb[3]);
+        pd[1] = pk2(vb[4], vb[5]);
+        own0 = nown0;
+        own1 = nown1;
+    }
+}
+
+// The walker of a wavelet over one strip: inner strips (most) run an instance
+// without wrapped columns.
+template <typename T, int WAV, int NB, int LAY, class Emit>
+__device__ __forceinline__ void walk_rows(const SceneArgs &s, const LaneCols &c, int64_t x0, int m_s, int m_e, int b0,
+                                          Emit &out) {
+    if (LAY != kPairs && strip_inner(x0, s.W)) {
+        if (WAV == 0)
+            haar_rows<T, NB, LAY, LAY != kPairs>(s, c, m_s, m_e, b0, out);
+        else
+            d4_rows<T, NB, LAY, LAY != kPairs>(s, c, m_s, m_e, b0, out);
+    } else {
+        if (WAV == 0)
+            haar_rows<T, NB, LAY, false>(s, c, m_s, m_e, b0, out);
+        else
+            d4_rows<T, NB, LAY, false>(s, c, m_s, m_e, b0, out);
     }
 }
 
 // ------------------------------------------------------------------ direct emitter
 
-// Every lane writes its own 4 pixels to global memory.  ALT: the W % 4 == 2
-// instance (even rows vectorised, odd rows through store4_shifted).
-template <bool ALT>
-struct DirectEmit {
-    static constexpr bool kAllLanes = ALT;
-    const SceneArgs &s;
-    const LaneCols &c;
-    int b0, lane;
-    bool a4, a4e, alt;
+// Writes the lane's 4 fused pixels x .. x+3 of one band row at p (the address
+// of column x).  `odd`: an odd image row; under kShift it starts 2 pixels past
+// a 4-pixel boundary, and every lane but the first writes the aligned vector
+// x-2 .. x+1, taking pixels x-2, x-1 from its left neighbour; lane 0 writes
+// x, x+1 and the last lane of the strip (x + 4 >= W or lane 31) also
+// x+2, x+3.  Under kShift every lane of the warp calls it (warp shuffles).
+template <int LAY>
+__device__ __forceinline__ void store_f32(float *p, const LaneCols &c, int lane, bool odd, const float *v) {
+    if (LAY == kShift && odd) {
+        const float p2 = __shfl_up_sync(0xffffffffu, v[2], 1);
+        const float p3 = __shfl_up_sync(0xffffffffu, v[3], 1);
+        if (c.active) {
+            if (lane > 0)
+                __stcs(reinterpret_cast<float4 *>(p - 2), make_float4(p2, p3, v[0], v[1]));
+            else
+                __stcs(reinterpret_cast<float2 *>(p), make_float2(v[0], v[1]));
+            if (c.two && c.last) __stcs(reinterpret_cast<float2 *>(p + 2), make_float2(v[2], v[3]));
+        }
+        return;
+    }
+    if (!c.active) return;
+    if (LAY == kVec || (LAY == kShift && c.two)) {
+        __stcs(reinterpret_cast<float4 *>(p), make_float4(v[0], v[1], v[2], v[3]));
+    } else {
+        __stcs(reinterpret_cast<float2 *>(p), make_float2(v[0], v[1]));
+        if (c.two) __stcs(reinterpret_cast<float2 *>(p + 2), make_float2(v[2], v[3]));
+    }
+}
+// The same for the 4 rounded pixels in w.
+template <int LAY>
+__device__ __forceinline__ void store_u8(uint8_t *p, const LaneCols &c, int lane, bool odd, uint32_t w) {
+    if (LAY == kShift && odd) {
+        const uint32_t pw = __shfl_up_sync(0xffffffffu, w, 1);
+        if (c.active) {
+            if (lane > 0)
+                __stcs(reinterpret_cast<unsigned int *>(p - 2), __byte_perm(pw, w, 0x5432u));
+            else
+                __stcs(reinterpret_cast<unsigned short *>(p), (unsigned short)(w & 0xffffu));
+            if (c.two && c.last) __stcs(reinterpret_cast<unsigned short *>(p + 2), (unsigned short)(w >> 16));
+        }
+        return;
+    }
+    if (!c.active) return;
+    if (LAY == kVec || (LAY == kShift && c.two)) {
+        __stcs(reinterpret_cast<unsigned int *>(p), w);
+    } else {
+        __stcs(reinterpret_cast<unsigned short *>(p), (unsigned short)(w & 0xffffu));
+        if (c.two) __stcs(reinterpret_cast<unsigned short *>(p + 2), (unsigned short)(w >> 16));
+    }
+}
 
-    __device__ __forceinline__ void band(int b, int64_t m, const float *v0, const float *v1, float, float) const {
-        const int64_t W = s.W, HW = s.out_plane, y = 2 * (m - s.m_lo);
-        if constexpr (ALT) {
-            OutPtrs o{s.out_f32 ? s.out_f32 + (int64_t)(b0 + b) * HW : nullptr,
-                      s.out_u8 ? s.out_u8 + (int64_t)(b0 + b) * HW : nullptr};
-            if (c.active) store4(o, y * W + c.x, a4e, c.two, v0);
-            if (alt)
-                store4_shifted(o, (y + 1) * W + c.x, lane, c.active, c.two, c.last, v1);
-            else if (c.active)
-                store4(o, (y + 1) * W + c.x, a4, c.two, v1);
-        } else if (c.active) {
-            OutPtrs o{s.out_f32 ? s.out_f32 + (int64_t)(b0 + b) * HW : nullptr,
-                      s.out_u8 ? s.out_u8 + (int64_t)(b0 + b) * HW : nullptr};
-            store4(o, y * W + c.x, a4, c.two, v0);
-            store4(o, (y + 1) * W + c.x, a4, c.two, v1);
+// Output addresses of a lane, running: the band's fused pixels (row 2m, column
+// x) of the band in hand, stepped by a plane per band and by two rows less
+// the planes stepped at the end of an MS row.
+struct OutRun {
+    float *f;
+    uint8_t *u;
+    bool hf, hu;  // which outputs are wanted (the other's address is not used)
+    __device__ __forceinline__ OutRun(const SceneArgs &s, const LaneCols &c, int b0, int m_s)
+        : hf(s.out_f32 != nullptr), hu(s.out_u8 != nullptr) {
+        const int64_t off = (int64_t)b0 * s.out_plane + (int64_t)(2 * (m_s - s.m_lo)) * s.W + c.x;
+        f = s.out_f32 + off;
+        u = s.out_u8 + off;
+    }
+    __device__ __forceinline__ void next_row(int64_t step) {
+        f += step;
+        u += step;
+    }
+};
+
+// Every lane writes its own 4 pixels to global memory.  kVec: 4-pixel
+// vectors; kShift: even rows as vectors (the lane at x = W-2 pairs), odd rows
+// through store4_shifted; kPairs: pixel pairs.
+template <int LAY, int MODE>
+struct DirectEmit {
+    static constexpr bool kAllLanes = LAY == kShift;
+    static constexpr int kMode = MODE;
+    const LaneCols &c;
+    OutRun o;
+    int64_t plane;
+    int W, lane;
+
+    __device__ __forceinline__ DirectEmit(const SceneArgs &s, const LaneCols &cc, int b0, int m_s, int ln)
+        : c(cc), o(s, cc, b0, m_s), plane(s.out_plane), W((int)s.W), lane(ln) {}
+
+    template <typename M>
+    __device__ __forceinline__ void band(int, const float *v0, const float *v1, M, M) {
+        if (o.hf) {
+            store_f32<LAY>(o.f, c, lane, false, v0);
+            store_f32<LAY>(o.f + W, c, lane, true, v1);
+            o.f += plane;
+        }
+        if (o.hu) {
+            store_u8<LAY>(o.u, c, lane, false, pack4u8(v0));
+            store_u8<LAY>(o.u + W, c, lane, true, pack4u8(v1));
+            o.u += plane;
         }
     }
-    __device__ __forceinline__ void row_end(int64_t, const float *, const float *) const {}
+    template <int NB>
+    __device__ __forceinline__ void row_end(int, uint32_t, uint32_t) {
+        o.next_row(2 * (int64_t)W - NB * plane);
+    }
 };
 
 // One warp strip: 128 PAN columns from x0, MS rows [m_s, m_e), bands
-// [b0, b0 + NB) (nb of them live), written directly.
-template <typename T, int WAV, int NB, bool ALT>
-__device__ __forceinline__ void direct_item(const SceneArgs &s, int64_t x0, int64_t m_s, int64_t m_e,
-                                            int b0, int nb, int lane) {
+// [b0, b0 + NB), written directly.
+template <typename T, int WAV, int NB, int LAY, int MODE>
+__device__ __forceinline__ void direct_item(const SceneArgs &s, int64_t x0, int m_s, int m_e, int b0, int lane) {
     const LaneCols c = lane_cols(x0, lane, s.W);
-    const bool a4 = s.a4 != 0;
-    const bool alt = ALT && !a4 && s.alt != 0;  // even rows aligned, odd rows 2 pixels past
-    // Vector path on even rows; the last lane (x = W-2) keeps the wrapped pair loads
-    // and 2-pixel stores there.
-    const bool a4e = a4 || (alt && c.two);
-    DirectEmit<ALT> out{s, c, b0, lane, a4, a4e, alt};
-    if (WAV == 0)
-        haar_rows<T, NB>(s, c, a4e, a4, m_s, m_e, b0, nb, out);
-    else
-        d4_rows<T, NB>(s, c, a4e, a4, m_s, m_e, b0, nb, out);
+    DirectEmit<LAY, MODE> out(s, c, b0, m_s, lane);
+    walk_rows<T, WAV, NB, LAY>(s, c, x0, m_s, m_e, b0, out);
 }
 
 // Geometry of a scene's work items: strips of 128 PAN columns times runs of R MS rows.
@@ -454,21 +827,13 @@ __host__ __device__ inline ItemGrid item_grid(int64_t H, int64_t W, int R) {
     return g;
 }
 
-// Runs work item `item` of a scene: WAV < 0 selects the wavelet at run time
-// (batched kernel), 0 / 1 fixes Haar / D4 at compile time.  ALT compiles the
-// shifted-row store path of widths W % 4 == 2 (taken when s.alt is set);
-// without it such scenes use the scalar edge path.
-template <typename T, int WAV, int NB, bool ALT = false>
-__device__ __forceinline__ void run_item(const SceneArgs &s, int64_t item, int64_t strips_x, int R,
-                                         int b0, int nb, int lane) {
+// Runs work item `item` of a scene on the walkers of one row layout.
+template <typename T, int WAV, int NB, int LAY, int MODE>
+__device__ __forceinline__ void run_item(const SceneArgs &s, int64_t item, int64_t strips_x, int R, int b0, int lane) {
     const int64_t sx = item % strips_x, sy = item / strips_x;
-    const int64_t x0 = sx * kWarpCols;
-    const int64_t m_s = s.m_lo + sy * R;
-    const int64_t m_e = min(m_s + (int64_t)R, (int64_t)s.m_hi);
-    if (WAV == 0 || (WAV < 0 && s.wavelet == 0))
-        direct_item<T, 0, NB, ALT>(s, x0, m_s, m_e, b0, nb, lane);
-    else
-        direct_item<T, 1, NB, ALT>(s, x0, m_s, m_e, b0, nb, lane);
+    const int m_s = s.m_lo + (int)(sy * R);
+    const int m_e = min(m_s + R, s.m_hi);
+    direct_item<T, WAV, NB, LAY, MODE>(s, sx * kWarpCols, m_s, m_e, b0, lane);
 }
 
 }  // namespace dwtfuse
