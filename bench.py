@@ -91,6 +91,9 @@ KNOWN_TRAFFIC: dict[str, float] = {
     # walkers with paired FP32 and running addresses:
     # read 708,970,496 + write 8,006,513,664 (mean of 2 launches)
     "686a90346174": 8715484160.0,
+    # row heights per launch, scalar synthesis where registers are short:
+    # read 709,261,440 + write 8,006,737,536 (mean of 2 launches)
+    "4ac0e872cfb0": 8715998976.0,
 }
 KERNEL_SOURCES = ("fuse_tile.cuh", "fuse_metrics.cu", "metric_q.cuh", "tmem.cuh")
 

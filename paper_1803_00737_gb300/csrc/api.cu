@@ -155,16 +155,16 @@ int make_scene(const void *pan, const void *const *ms, int bands, int64_t H, int
     return DWTFUSE_OK;
 }
 
-// Scene table of a batched launch.  A scene whose rows are 2 pixels off the
+// Scene table of a batched launch (its work items are laid out per launch, by
+// launch_fuse_batched).  A scene whose rows are 2 pixels off the
 // 16-byte grid on every other row (W % 4 == 2, aligned planes) is run by the
 // shifted-row item body, which holds at most kBatchAltMaxBands bands: with
 // more, its bands are split over two table entries (the same PAN read twice)
 // while the table has room, else it takes the plain pixel-pair body.
 int build_batch_table(const dwtfuse_scene *scenes, int n, int rows_per_item, BatchTable *t) {
     std::memset(t, 0, sizeof *t);
-    t->R = rows_per_item > 0 ? rows_per_item : kDefaultRows;
+    t->R = rows_per_item;
     const int knob = fwd_band_chunk();
-    int64_t acc = 0;
     int k = 0;
     for (int i = 0; i < n; ++i) {
         const dwtfuse_scene &d = scenes[i];
@@ -173,7 +173,6 @@ int build_batch_table(const dwtfuse_scene *scenes, int n, int rows_per_item, Bat
         const int st = make_scene(d.pan, d.ms, d.bands, d.H, d.W, d.wavelet, d.in_dtype, d.out_f32, d.out_u8,
                                   kBatchMaxBands, &sa);
         if (st != DWTFUSE_OK) return st;
-        const ItemGrid g = item_grid(d.H, d.W, t->R);
         const bool alt = sa.alt && !sa.a4;
         // Band groups per entry: at most kBatchAltMaxBands on shifted rows, at
         // most the band-chunk knob when it is set; balanced groups.
@@ -198,14 +197,11 @@ int build_batch_table(const dwtfuse_scene *scenes, int n, int rows_per_item, Bat
                 if (e.out_u8) e.out_u8 += (int64_t)b0 * HW;
             }
             t->scenes[k] = e;
-            t->item_start[k] = acc;
-            t->strips_x[k] = g.strips_x;
-            acc += g.items;
+            t->strips_x[k] = (d.W + kWarpCols - 1) / kWarpCols;
             ++k;
         }
     }
     t->n = k;
-    t->item_start[k] = acc;
     return DWTFUSE_OK;
 }
 

@@ -480,17 +480,7 @@ cudaError_t launch_dwt2_staged(const DwtArgs &s, const DwtLaunch &d, cudaStream_
     const int64_t cap = (int64_t)sms * occ, rows = d.H / 2;
     const int64_t strips = (d.W + kDwtCols - 1) / kDwtCols;
     int R = d.rows;
-    if (R <= 0) {  // coefficient rows per CTA item that fill the last wave (+1: the D4 prologue)
-        double best = 1e300;
-        for (int r = 16; r <= 128; ++r) {
-            const int64_t n = strips * ((rows + r - 1) / r);
-            const double cost = (double)((n + cap - 1) / cap) * (r + 1);
-            if (cost <= best) {
-                best = cost;
-                R = r;
-            }
-        }
-    }
+    if (R <= 0) R = balanced_rows(strips, rows, cap, 128);
     const int64_t items = strips * ((rows + R - 1) / R);
     const unsigned grid = (unsigned)(items < cap ? items : cap);
     if (grid == 0) return cudaSuccess;
@@ -519,7 +509,7 @@ cudaError_t launch_dwt2(const DwtLaunch &d, cudaStream_t stream) {
     e = sm_count(&sms);
     if (e != cudaSuccess) return e;
     const int64_t cap = (int64_t)sms * occ;
-    int R = d.rows > 0 ? d.rows : balanced_rows(d.H, d.W, cap * kDwtWarps);
+    int R = d.rows > 0 ? d.rows : balanced_rows((d.W + kWarpCols - 1) / kWarpCols, d.H / 2, cap * kDwtWarps);
     const ItemGrid g = item_grid(d.H, d.W, R);
     const int64_t need = (g.items + kDwtWarps - 1) / kDwtWarps;
     const unsigned grid = (unsigned)(need < cap ? need : cap);

@@ -7,11 +7,20 @@ namespace dwtfuse {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kAltMaxBands = 6;  // widest band chunk of the shifted-row instance
+// Shifted rows: neighbouring strips complete each other's sectors, and short
+// items bring them there close together (rows per item 4 against the balanced
+// height: 16384 x 16382 x 6 float + uint8 1948 -> 1804 us, 5000 x 5002 x 6 174
+// -> 160, 3736 x 4070 x 3 49.2 -> 46.2; aligned rows gain nothing: 8192^2 x 8
+// float 520 -> 526).
+constexpr int kShiftRows = 4;
 
-// PAN rows one row ahead for up to 4 bands (3736 x 4070 x 3, uint8: 58 -> 53.5
-// us a call; 8 bands, which then spill: 185 -> 192 us at 7480 x 8140).
-template <int NB>
-constexpr int kFwdMode = NB <= 4 ? kAheadPan : 0;
+// Walker mode (paired / scalar FP32 and loads ahead, us a call): up to 4 bands
+// PAN one row ahead (3736 x 4070 x 3 uint8 58 -> 53.5); more bands scalar
+// columns (8192^2 x 8 uint8 to float + uint8 502 -> 491, to uint8 alone 205 ->
+// 211), floats scalar rows too (8192^2 x 8 522 -> 493, 6 bands on shifted rows
+// 405 -> 398).
+template <typename T, int NB>
+constexpr int kFwdMode = NB <= 4 ? kAheadPan : (sizeof(T) == 4 ? kScalarCol | kScalarRow : kScalarCol);
 
 // Single scene, bands [b0, b0 + NB).  Each warp takes work items
 // warp, warp + total_warps, ... (grid sized to the resident capacity).
@@ -23,7 +32,7 @@ fuse_fwd_kernel(const __grid_constant__ SceneArgs s, int b0, int64_t strips_x, i
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t)gridDim.x * kWarps;
     for (int64_t it = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5); it < items; it += nwarps)
-        run_item<T, WAV, NB, LAY, kFwdMode<NB>>(s, it, strips_x, R, b0, lane);
+        run_item<T, WAV, NB, LAY, kFwdMode<T, NB>>(s, it, strips_x, R, b0, lane);
 }
 
 // ------------------------------------------------------------------ host side
@@ -87,7 +96,11 @@ cudaError_t launch_fuse(const SceneArgs &s, int R, int blocks_per_sm, cudaStream
         const int64_t cap = (int64_t)sms * occ;
         // Items cover the MS rows [m_lo, m_hi) (all of them for a whole scene).
         const int64_t rows2 = 2 * (int64_t)(s.m_hi - s.m_lo);
-        int Rl = R > 0 ? R : balanced_rows(rows2, s.W, cap * kWarps);
+        int Rl = R;
+        if (Rl <= 0) {
+            Rl = balanced_rows((s.W + kWarpCols - 1) / kWarpCols, rows2 / 2, cap * kWarps);
+            if (alt && Rl > kShiftRows) Rl = kShiftRows;
+        }
         const ItemGrid g = item_grid(rows2, s.W, Rl);
         const int64_t need = (g.items + kWarps - 1) / kWarps;
         const unsigned grid = (unsigned)(need < cap ? need : cap);

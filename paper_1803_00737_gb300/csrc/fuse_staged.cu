@@ -48,8 +48,12 @@ __device__ __forceinline__ void bulk_wait_read() {
 
 template <int NB>
 struct StagedEmit {
-    static constexpr bool kAllLanes = true;  // every lane reaches the row barrier
-    static constexpr int kMode = 0;
+    // Up to 4 bands: the next row's inputs loaded ahead (8192^2 x 3 208 -> 184
+    // us).  More: scalar synthesis, and the uint8 pixels stored after the
+    // float rows' copies are issued, behind the row barrier (16384^2 x 6 float
+    // + uint8 1388 -> 1340 us; with 3 bands that costs 208 -> 217).
+    static constexpr bool kLate = NB > 4;
+    static constexpr int kMode = NB > 4 ? kScalarCol | kScalarRow : kAheadPan | kAheadMs;
     const SceneArgs &s;
     const LaneCols &c;
     float *buf;    // two slots of [NB][2][kStCols] floats
@@ -59,20 +63,30 @@ struct StagedEmit {
     int *rowc;     // the CTA's row count: row k fills slot k & 1
     bool hu;       // uint8 output wanted
     uint8_t *u;    // its band b0, the current MS row's first image row, column x
+    uint32_t w8[kLate ? NB : 1][2];  // kLate: the row's uint8 words
 
     __device__ __forceinline__ float *slot() const { return buf + (*rowc & 1) * (NB * 2 * kStCols); }
 
     template <typename M>
     __device__ __forceinline__ void band(int b, const float *v0, const float *v1, M, M) {
-        u += b ? s.out_plane : 0;
+        if (kLate) {
+            if (hu) {
+                w8[kLate ? b : 0][0] = pack4u8(v0);
+                w8[kLate ? b : 0][1] = pack4u8(v1);
+            }
+        } else {
+            u += b ? s.out_plane : 0;
+        }
         if (!c.active) return;
         float *row = slot() + b * 2 * kStCols + (c.x - (int)X0);
         *reinterpret_cast<float4 *>(row) = make_float4(v0[0], v0[1], v0[2], v0[3]);
         *reinterpret_cast<float4 *>(row + kStCols) = make_float4(v1[0], v1[1], v1[2], v1[3]);
-        if (hu) {
-            store_u8<kVec>(u, c, 0, false, pack4u8(v0));
-            store_u8<kVec>(u + s.W, c, 0, true, pack4u8(v1));
-        }
+        if (!kLate && hu) store_rows(u, pack4u8(v0), pack4u8(v1));
+    }
+
+    __device__ __forceinline__ void store_rows(uint8_t *q, uint32_t w0, uint32_t w1) const {
+        store_u8<kVec>(q, c, 0, false, w0);
+        store_u8<kVec>(q + s.W, c, 0, true, w1);
     }
 
     template <int>
@@ -91,7 +105,19 @@ struct StagedEmit {
                          : "memory");
             asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
         }
-        u += 2 * s.W - (NB - 1) * s.out_plane;
+        if (kLate) {
+            if (hu) {
+                uint8_t *q = u;
+#pragma unroll
+                for (int b = 0; b < (kLate ? NB : 1); ++b) {
+                    store_rows(q, w8[b][0], w8[b][1]);
+                    q += s.out_plane;
+                }
+            }
+            u += 2 * s.W;
+        } else {
+            u += 2 * s.W - (NB - 1) * s.out_plane;
+        }
         ++*rowc;
     }
 };
@@ -191,17 +217,7 @@ cudaError_t launch_fuse_staged(const SceneArgs &s, int R, cudaStream_t stream) {
         const int64_t rows = (int64_t)(s.m_hi - s.m_lo);
         const int64_t strips = staged_strips(s.W);
         int Rl = R;
-        if (Rl <= 0) {  // MS rows per CTA item that fill the last wave (+1: the D4 prologue row)
-            double best = 1e300;
-            for (int r = 16; r <= 128; ++r) {
-                const int64_t n = strips * ((rows + r - 1) / r);
-                const double cost = (double)((n + capc - 1) / capc) * (r + 1);
-                if (cost <= best) {
-                    best = cost;
-                    Rl = r;
-                }
-            }
-        }
+        if (Rl <= 0) Rl = balanced_rows(strips, rows, capc, 128);
         const int64_t items = strips * ((rows + Rl - 1) / Rl);
         const unsigned grid = (unsigned)(items < capc ? items : capc);
         if (grid == 0) continue;

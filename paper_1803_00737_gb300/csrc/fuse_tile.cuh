@@ -464,12 +464,13 @@ __device__ __forceinline__ float ms_f(float v) { return v; }
 //   kAheadPan, kAheadMs  load the next MS row's PAN rows / MS values one row
 //                        ahead (raw words and bytes; they stay in registers
 //                        for a whole row)
-//   kScalarCol           column synthesis in scalar FP32 (its constants are
-//                        immediates; the paired form holds 8 registers of
-//                        them, which spill in the scoring kernel)
-// Measured per kernel (see there): ahead pays where few bands leave registers
-// free, and costs where the walker then spills.
-enum : int { kAheadPan = 1, kAheadMs = 2, kScalarCol = 4 };
+//   kScalarCol, kScalarRow  column / row synthesis in scalar FP32 (its
+//                        constants are immediates; the paired form holds 8 and
+//                        4 registers of them)
+// Chosen per kernel by measurement (see there): loads ahead pay where few bands
+// leave registers free, paired FP32 where instructions bound the kernel and
+// nothing spills.
+enum : int { kAheadPan = 1, kAheadMs = 2, kScalarCol = 4, kScalarRow = 8 };
 
 // Haar (Eq. 1-2, 11-12).
 template <typename T, int NB, int LAY, bool INNER, class Emit>
@@ -556,6 +557,11 @@ __device__ __forceinline__ void d4_rows(const SceneArgs &s, const LaneCols &c, i
         const float eA = fmaf(gain, ms_f(mv[0]), -ll[0]);
         const float eB = fmaf(gain, ms_f(mv[1]), -ll[1]);
         const float eC = fmaf(gain, ms_f(mv[2]), -ll[2]);
+        if constexpr ((Emit::kMode & kScalarRow) != 0) {
+            lo = pk2(fmaf(kH2, eA, kH0 * eB), fmaf(kH3, eA, kH1 * eB));
+            hi = pk2(fmaf(kH2, eB, kH0 * eC), fmaf(kH3, eB, kH1 * eC));
+            return;
+        }
         const f32x2 bb = pk2(eB, eB);
         lo = fma2(h23, pk2(eA, eA), mul2(h01, bb));
         hi = fma2(h23, bb, mul2(h01, pk2(eC, eC)));

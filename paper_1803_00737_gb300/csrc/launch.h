@@ -13,7 +13,7 @@ constexpr int kChunkBands = 8;     // bands per single-scene launch (more = seve
 constexpr int kBatchMaxBands = 8;
 constexpr int kBatchAltMaxBands = 6;  // bands of the batched shifted-row (W % 4 == 2) item body  // bands per scene in the batched kernel
 constexpr int kMaxScenes = 128;    // scenes per batched launch
-constexpr int kDefaultRows = 32;   // MS rows per warp work item (batched default)
+constexpr int kDefaultRows = 32;   // most MS rows per warp work item of a batched launch by default
 constexpr size_t kQueueBytes = 16; // queue counter (8) + status word (4) + pad
 constexpr int kStagedMaxBands = 6; // bands per launch of the staged forward (fuse_staged.cu)
 
@@ -21,7 +21,7 @@ constexpr int kStagedMaxBands = 6; // bands per launch of the staged forward (fu
 // parameter block (< 32 KB), so a captured graph owns its own copy.
 struct BatchTable {
     int32_t n;
-    int32_t R;
+    int32_t R;  // MS rows per item (0: chosen per launch)
     int64_t item_start[kMaxScenes + 1];
     int64_t strips_x[kMaxScenes];
     SceneArgs scenes[kMaxScenes];
@@ -62,15 +62,18 @@ struct MetricLaunch {
 constexpr int kFuseMetricsMaxBands = 8;
 
 // MS rows per work item that balance the last wave of a grid of `warps`
-// warps: minimises ceil(items / warps) * (R + 1) over R in [16, 64] (the +1
-// is the D4 prologue row of every item); ties go to the taller item.
-inline int balanced_rows(int64_t H, int64_t W, int64_t warps) {
-    int best = kDefaultRows;
+// workers over `strips` column strips of `rows` MS rows: minimises
+// ceil(items / warps) * (R + 1) over R in [1, hi] (the +1 is the D4 prologue
+// row of every item); ties go to the taller item.  Scenes too small for one
+// 16-row item per worker get shorter ones, down to single rows (a floor of 16
+// left most of the GPU idle there: a 512 x 512 scene ran in 8 CTAs, 31 us a
+// kernel; 2048 x 2050 inverse transform 12.1 -> 10.4 us a call).
+inline int balanced_rows(int64_t strips, int64_t rows, int64_t warps, int hi = 64) {
+    int best = 1;
     double best_cost = 1e300;
-    for (int R = 16; R <= 64; ++R) {
-        const ItemGrid g = item_grid(H, W, R);
-        const int64_t waves = (g.items + warps - 1) / warps;
-        const double cost = (double)waves * (double)(R + 1);
+    for (int R = 1; R <= hi; ++R) {
+        const int64_t items = strips * ((rows + R - 1) / R);
+        const double cost = (double)((items + warps - 1) / warps) * (double)(R + 1);
         if (cost <= best_cost) {
             best_cost = cost;
             best = R;

@@ -27,14 +27,13 @@ import threading
 from dataclasses import dataclass
 from typing import Callable, Iterable
 
-ROWS = (8, 16, 24, 32, 48, 64)
+ROWS = (0, 8, 16, 24, 32, 48)  # 0 = the library's rule on the table's sizes
 BLOCKS = (0,)  # 0 = as many CTAs per SM as fit
 FWD_CHUNKS = (0, 6, 4)  # 0 = library default (8 bands per launch, 6 on shifted rows)
 BWD_CHUNKS = (0, 4)     # 0 = library default (8)
 # Bumped when the kernels behind the knobs change enough that cached choices
-# may no longer be the fastest (3: TMEM scoring kernel, narrow batched
-# instance).
-CACHE_VERSION = 3
+# may no longer be the fastest (4: paired-FP32 walkers, batched default rows).
+CACHE_VERSION = 4
 
 _lock = threading.Lock()
 
