@@ -305,6 +305,25 @@ int dwtfuse_fuse_batched(const dwtfuse_scene *scenes, int n, void *workspace, si
                          int rows_per_item, int blocks_per_sm, void *stream);
 
 /*
+ * dwtfuse_fuse_batched over n scenes of one shape whose images lie one after
+ * the other (a batch tensor): pan [n][H][W], ms [n][bands][H/2][W/2], outputs
+ * [n][bands][H][W].  The scene table is laid out here instead of by the
+ * caller; any n >= 1 (more than DWTFUSE_MAX_SCENES run as several calls).
+ * Results, errors and the other arguments as dwtfuse_fuse_batched.
+ */
+int dwtfuse_fuse_batched_uniform(const void *pan, const void *ms, int64_t n, int bands, int64_t H, int64_t W,
+                                 int wavelet, int in_dtype, float *out_f32, uint8_t *out_u8, void *workspace,
+                                 size_t ws_bytes, int rows_per_item, int blocks_per_sm, void *stream);
+
+/*
+ * dwtfuse_fuse_backward_batched in the same layout: grad_out [n][bands][H][W],
+ * grad_pan [n][H][W], grad_ms [n][bands][H/2][W/2].
+ */
+int dwtfuse_fuse_backward_batched_uniform(const float *grad_out, int64_t n, int bands, int64_t H, int64_t W,
+                                          int wavelet, float *grad_pan, float *grad_ms, void *workspace,
+                                          size_t ws_bytes, void *stream);
+
+/*
  * Reads (synchronously, on `stream`) the device status word of a batched
  * workspace: DWTFUSE_OK, or the first device-side error recorded.  With
  * workspace = NULL it reads the status word of the last

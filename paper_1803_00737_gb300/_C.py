@@ -80,6 +80,8 @@ _SIGS = {
     "dwtfuse_fuse_backward_batched": (_i, [ctypes.POINTER(GradScene), _i, _vp, _sz, _vp]),
     "dwtfuse_batched_workspace_size": (_sz, []),
     "dwtfuse_fuse_batched": (_i, [ctypes.POINTER(Scene), _i, _vp, _sz, _i, _i, _vp]),
+    "dwtfuse_fuse_batched_uniform": (_i, [_vp, _vp, _i64, _i, _i64, _i64, _i, _i, _vp, _vp, _vp, _sz, _i, _i, _vp]),
+    "dwtfuse_fuse_backward_batched_uniform": (_i, [_vp, _i64, _i, _i64, _i64, _i, _vp, _vp, _vp, _sz, _vp]),
     "dwtfuse_get_last_device_status": (_i, [_vp, _vp]),
     "dwtfuse_set_rows_per_item": (_i, [_i]),
     "dwtfuse_set_band_chunks": (_i, [_i, _i]),
@@ -108,6 +110,8 @@ _lib = None
 def lib() -> ctypes.CDLL:
     """The loaded libdwtfuse.so (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB):
@@ -173,20 +177,23 @@ def _bands(ms) -> list[torch.Tensor]:
     return list(ms)
 
 
+def _band_ptrs(ms, dtype: torch.dtype, h: int, w: int):
+    """Pointer array of the bands of one dense (B, h, w) GPU tensor of the given
+    type, from its base address; None for anything else (the callers then look
+    at band by band, and say what is wrong)."""
+    if (isinstance(ms, torch.Tensor) and ms.dim() == 3 and ms.dtype == dtype and ms.is_cuda
+            and ms.is_contiguous() and ms.shape[0] > 0 and ms.shape[1] == h and ms.shape[2] == w and h > 0 and w > 0):
+        p, step = ms.data_ptr(), h * w * ms.element_size()
+        return (_vp * ms.shape[0])(*range(p, p + ms.shape[0] * step, step))
+    return None
+
+
 def dwtfuse_fuse(pan: torch.Tensor, ms, wavelet: int, out_f32: torch.Tensor | None = None,
                  out_u8: torch.Tensor | None = None, stream=None) -> None:
     """Fused forward into caller-provided outputs (see dwtfuse_fuse in dwtfuse.h)."""
-    bands = _bands(ms)
-    H, W = pan.shape
+    n, H, W, ptrs = _fuse_score_args(pan, ms, out_f32, out_u8)
     code = _dtype_code(pan, "pan")
-    ptrs = (_vp * len(bands))(*[_dev(m, f"ms[{b}]") for b, m in enumerate(bands)])
-    for b, m in enumerate(bands):
-        if m.dtype != pan.dtype or tuple(m.shape) != (H // 2, W // 2):
-            raise ValueError(f"ms[{b}] must be {pan.dtype} of shape ({H // 2}, {W // 2})")
-    for name, o, dt in (("out_f32", out_f32, torch.float32), ("out_u8", out_u8, torch.uint8)):
-        if o is not None and (o.dtype != dt or tuple(o.shape) != (len(bands), H, W)):
-            raise ValueError(f"{name} must be {dt} of shape ({len(bands)}, {H}, {W})")
-    st = lib().dwtfuse_fuse(_dev(pan, "pan"), ptrs, len(bands), H, W, int(wavelet), code,
+    st = lib().dwtfuse_fuse(_dev(pan, "pan"), ptrs, n, H, W, int(wavelet), code,
                             _dev(out_f32, "out_f32") if out_f32 is not None else None,
                             _dev(out_u8, "out_u8") if out_u8 is not None else None,
                             _stream(stream))
@@ -275,13 +282,17 @@ def dwtfuse_fuse_backward(grad_out: torch.Tensor, wavelet: int, grad_pan: torch.
     B, H, W = grad_out.shape
     if grad_out.dtype != torch.float32 or grad_pan.dtype != torch.float32:
         raise TypeError("gradients must be float32")
-    gms = _bands(grad_ms)
-    if len(gms) != B:
+    ptrs = _band_ptrs(grad_ms, torch.float32, H // 2, W // 2)
+    if ptrs is None:
+        gms = _bands(grad_ms)
+        if len(gms) != B:
+            raise ValueError("one grad_ms buffer per band")
+        for b, g in enumerate(gms):
+            _need(g, (H // 2) * (W // 2), torch.float32, f"grad_ms[{b}]")
+        ptrs = (_vp * B)(*[_dev(g, f"grad_ms[{b}]") for b, g in enumerate(gms)])
+    if len(ptrs) != B:
         raise ValueError("one grad_ms buffer per band")
     _need(grad_pan, H * W, torch.float32, "grad_pan")
-    for b, g in enumerate(gms):
-        _need(g, (H // 2) * (W // 2), torch.float32, f"grad_ms[{b}]")
-    ptrs = (_vp * B)(*[_dev(g, f"grad_ms[{b}]") for b, g in enumerate(gms)])
     st = lib().dwtfuse_fuse_backward(_dev(grad_out, "grad_out"), B, H, W, int(wavelet),
                                      _dev(grad_pan, "grad_pan"), ptrs, _stream(stream))
     _check(st, "dwtfuse_fuse_backward")
@@ -314,6 +325,43 @@ def dwtfuse_fuse_backward_batched(scenes: list[GradScene], workspace: torch.Tens
                                              workspace.numel() * workspace.element_size(),
                                              _stream(stream))
     _check(st, "dwtfuse_fuse_backward_batched")
+
+
+def dwtfuse_fuse_batched_uniform(pan: torch.Tensor, ms: torch.Tensor, wavelet: int,
+                                 out_f32: torch.Tensor | None, out_u8: torch.Tensor | None,
+                                 workspace: torch.Tensor, rows_per_item: int = 0, blocks_per_sm: int = 0,
+                                 stream=None) -> None:
+    """dwtfuse_fuse_batched over dense batch tensors: pan (N, H, W), ms
+    (N, B, H/2, W/2), outputs (N, B, H, W) (see dwtfuse.h)."""
+    N, H, W = pan.shape
+    B = ms.shape[1]
+    if ms.dtype != pan.dtype or tuple(ms.shape) != (N, B, H // 2, W // 2):
+        raise ValueError(f"ms must be {pan.dtype} of shape ({N}, bands, {H // 2}, {W // 2})")
+    for name, o, dt in (("out_f32", out_f32, torch.float32), ("out_u8", out_u8, torch.uint8)):
+        if o is not None and (o.dtype != dt or tuple(o.shape) != (N, B, H, W)):
+            raise ValueError(f"{name} must be {dt} of shape ({N}, {B}, {H}, {W})")
+    st = lib().dwtfuse_fuse_batched_uniform(
+        _dev(pan, "pan"), _dev(ms, "ms"), N, B, H, W, int(wavelet), _dtype_code(pan, "pan"),
+        _dev(out_f32, "out_f32") if out_f32 is not None else None,
+        _dev(out_u8, "out_u8") if out_u8 is not None else None, _dev(workspace, "workspace"),
+        workspace.numel() * workspace.element_size(), int(rows_per_item), int(blocks_per_sm), _stream(stream))
+    _check(st, "dwtfuse_fuse_batched_uniform")
+
+
+def dwtfuse_fuse_backward_batched_uniform(grad_out: torch.Tensor, wavelet: int, grad_pan: torch.Tensor,
+                                          grad_ms: torch.Tensor, workspace: torch.Tensor, stream=None) -> None:
+    """dwtfuse_fuse_backward_batched over dense batch tensors: grad_out
+    (N, B, H, W), grad_pan (N, H, W), grad_ms (N, B, H/2, W/2) (see dwtfuse.h)."""
+    N, B, H, W = grad_out.shape
+    for name, t, shape in (("grad_out", grad_out, (N, B, H, W)), ("grad_pan", grad_pan, (N, H, W)),
+                           ("grad_ms", grad_ms, (N, B, H // 2, W // 2))):
+        if t.dtype != torch.float32 or tuple(t.shape) != shape:
+            raise ValueError(f"{name} must be float32 of shape {shape}")
+    st = lib().dwtfuse_fuse_backward_batched_uniform(
+        _dev(grad_out, "grad_out"), N, B, H, W, int(wavelet), _dev(grad_pan, "grad_pan"),
+        _dev(grad_ms, "grad_ms"), _dev(workspace, "workspace"),
+        workspace.numel() * workspace.element_size(), _stream(stream))
+    _check(st, "dwtfuse_fuse_backward_batched_uniform")
 
 
 def dwtfuse_batched_workspace_size() -> int:
@@ -367,8 +415,11 @@ def dwtfuse_metrics_workspace_size() -> int:
 
 
 def _metric_args(fused: torch.Tensor, ms):
-    bands = _bands(ms)
     B, H, W = fused.shape
+    ptrs = _band_ptrs(ms, ms.dtype, H // 2, W // 2) if isinstance(ms, torch.Tensor) else None
+    if ptrs is not None and len(ptrs) == B:
+        return [ms], B, H, W, ptrs  # (the callers look at the first band's type only)
+    bands = _bands(ms)
     if len(bands) != B:
         raise ValueError("one MS band per fused band")
     for b, m in enumerate(bands):
@@ -392,16 +443,21 @@ def dwtfuse_metrics(fused: torch.Tensor, ms, pan: torch.Tensor, workspace: torch
 
 
 def _fuse_score_args(pan: torch.Tensor, ms, out_f32, out_u8):
-    bands = _bands(ms)
+    """(bands, H, W, band pointers) of a forward call, its MS bands and outputs checked."""
     H, W = pan.shape
-    ptrs = (_vp * len(bands))(*[_dev(m, f"ms[{b}]") for b, m in enumerate(bands)])
-    for b, m in enumerate(bands):
-        if m.dtype != pan.dtype or tuple(m.shape) != (H // 2, W // 2):
-            raise ValueError(f"ms[{b}] must be {pan.dtype} of shape ({H // 2}, {W // 2})")
+    _dtype_code(pan, "pan")
+    ptrs = _band_ptrs(ms, pan.dtype, H // 2, W // 2)
+    if ptrs is None:
+        bands = _bands(ms)
+        ptrs = (_vp * len(bands))(*[_dev(m, f"ms[{b}]") for b, m in enumerate(bands)])
+        for b, m in enumerate(bands):
+            if m.dtype != pan.dtype or tuple(m.shape) != (H // 2, W // 2):
+                raise ValueError(f"ms[{b}] must be {pan.dtype} of shape ({H // 2}, {W // 2})")
+    n = len(ptrs)
     for name, o, dt in (("out_f32", out_f32, torch.float32), ("out_u8", out_u8, torch.uint8)):
-        if o is not None and (o.dtype != dt or tuple(o.shape) != (len(bands), H, W)):
-            raise ValueError(f"{name} must be {dt} of shape ({len(bands)}, {H}, {W})")
-    return bands, H, W, ptrs
+        if o is not None and (o.dtype != dt or tuple(o.shape) != (n, H, W)):
+            raise ValueError(f"{name} must be {dt} of shape ({n}, {H}, {W})")
+    return n, H, W, ptrs
 
 
 def _out_device(out_device: torch.Tensor):
@@ -415,8 +471,8 @@ def dwtfuse_fuse_metrics(pan: torch.Tensor, ms, wavelet: int, out_f32: torch.Ten
                          stream=None) -> None:
     """Fused forward into the caller's outputs, then ERGAS, QNR, D_lambda, D_s
     of the uint8 product into out_device[0:4] (async; see dwtfuse.h)."""
-    bands, H, W, ptrs = _fuse_score_args(pan, ms, out_f32, out_u8)
-    st = lib().dwtfuse_fuse_metrics(_dev(pan, "pan"), ptrs, len(bands), H, W, int(wavelet),
+    n, H, W, ptrs = _fuse_score_args(pan, ms, out_f32, out_u8)
+    st = lib().dwtfuse_fuse_metrics(_dev(pan, "pan"), ptrs, n, H, W, int(wavelet),
                                     _dtype_code(pan, "pan"),
                                     _dev(out_f32, "out_f32") if out_f32 is not None else None,
                                     _dev(out_u8, "out_u8"), _dev(workspace, "workspace"),
@@ -428,8 +484,8 @@ def dwtfuse_fuse_metrics(pan: torch.Tensor, ms, wavelet: int, out_f32: torch.Ten
 def dwtfuse_fuse_and_score(pan: torch.Tensor, ms, wavelet: int, out_f32: torch.Tensor | None,
                            out_u8: torch.Tensor, workspace: torch.Tensor, stream=None) -> None:
     """First half of dwtfuse_fuse_metrics: the forward that scores its product."""
-    bands, H, W, ptrs = _fuse_score_args(pan, ms, out_f32, out_u8)
-    st = lib().dwtfuse_fuse_and_score(_dev(pan, "pan"), ptrs, len(bands), H, W, int(wavelet),
+    n, H, W, ptrs = _fuse_score_args(pan, ms, out_f32, out_u8)
+    st = lib().dwtfuse_fuse_and_score(_dev(pan, "pan"), ptrs, n, H, W, int(wavelet),
                                       _dtype_code(pan, "pan"),
                                       _dev(out_f32, "out_f32") if out_f32 is not None else None,
                                       _dev(out_u8, "out_u8"), _dev(workspace, "workspace"),
@@ -440,8 +496,8 @@ def dwtfuse_fuse_and_score(pan: torch.Tensor, ms, wavelet: int, out_f32: torch.T
 def dwtfuse_score_finish(ms, pan: torch.Tensor, out_u8: torch.Tensor, workspace: torch.Tensor,
                          out_device: torch.Tensor, stream=None) -> None:
     """Second half of dwtfuse_fuse_metrics: MS-resolution pass and reduction."""
-    bands, H, W, ptrs = _fuse_score_args(pan, ms, None, out_u8)
-    st = lib().dwtfuse_score_finish(ptrs, _dev(pan, "pan"), _dtype_code(pan, "pan"), len(bands), H, W,
+    n, H, W, ptrs = _fuse_score_args(pan, ms, None, out_u8)
+    st = lib().dwtfuse_score_finish(ptrs, _dev(pan, "pan"), _dtype_code(pan, "pan"), n, H, W,
                                     _dev(out_u8, "out_u8"), _dev(workspace, "workspace"),
                                     workspace.numel() * workspace.element_size(),
                                     _out_device(out_device), _stream(stream))

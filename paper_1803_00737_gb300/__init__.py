@@ -22,7 +22,7 @@ def fuse(pan: torch.Tensor, ms, wavelet: int, f32: bool = True, u8: bool = False
     for this scene class (tune.tune_fuse), if there is one.
     """
     from . import tune
-    bands = _C._bands(ms)
+    bands = ms if isinstance(ms, torch.Tensor) and ms.dim() == 3 else _C._bands(ms)
     H, W = pan.shape
     out_f = torch.empty((len(bands), H, W), dtype=torch.float32, device=pan.device) if f32 else None
     out_u = torch.empty((len(bands), H, W), dtype=torch.uint8, device=pan.device) if u8 else None

@@ -34,15 +34,27 @@ def fuse_batch(P: torch.Tensor, M: torch.Tensor, wavelet: int, out: torch.Tensor
             _C.dwtfuse_fuse(P[i], M[i], wavelet, out[i], None)
         return
     ws = torch.empty(_C.dwtfuse_batched_workspace_size(), dtype=torch.uint8, device=P.device)
+    # One table entry per scene is laid out in the library when the batch tensors are dense.
+    dense = (P.is_contiguous() and M.is_contiguous() and out.is_contiguous() and M.dtype == P.dtype
+             and tuple(M.shape) == (N, B, P.shape[1] // 2, P.shape[2] // 2)
+             and tuple(out.shape) == (N, B, *P.shape[1:]) and P.shape[0] == N)
     for i0 in range(0, N, _C.MAX_SCENES):
-        idx = range(i0, min(N, i0 + _C.MAX_SCENES))
-        scenes = [_C.make_scene(P[i], M[i], wavelet, out[i], None) for i in idx]
-        specs = [(P.shape[1], P.shape[2], B, wavelet)] * len(idx)
+        n = min(N - i0, _C.MAX_SCENES)
+        specs = [(P.shape[1], P.shape[2], B, wavelet)] * n
+
+        def scenes():
+            return [_C.make_scene(P[i], M[i], wavelet, out[i], None) for i in range(i0, i0 + n)]
+
         shape = _shape(tune.current_device_key() + "|" + tune.batched_class(specs),
-                       lambda: tune.tune_batched(scenes, specs, ws))
+                       lambda: tune.tune_batched(scenes(), specs, ws))
         rows, blocks = (shape.rows_per_item, shape.blocks_per_sm) if shape else (0, 0)
         with tune.using(tune.LaunchShape(0, 0, shape.fwd_chunk, 0) if shape else None):
-            _C.dwtfuse_fuse_batched(scenes, ws, rows, blocks)
+            if dense:
+                whole = n == N
+                _C.dwtfuse_fuse_batched_uniform(P if whole else P[i0:i0 + n], M if whole else M[i0:i0 + n],
+                                                wavelet, out if whole else out[i0:i0 + n], None, ws, rows, blocks)
+            else:
+                _C.dwtfuse_fuse_batched(scenes(), ws, rows, blocks)
 
 
 def fuse_batch_backward(g: torch.Tensor, wavelet: int, gp: torch.Tensor, gm: torch.Tensor) -> None:
@@ -60,6 +72,10 @@ def fuse_batch_backward(g: torch.Tensor, wavelet: int, gp: torch.Tensor, gm: tor
                    lambda: tune.tune_backward(g, wavelet, gp, gm))
     ws = torch.empty(_C.dwtfuse_batched_workspace_size(), dtype=torch.uint8, device=g.device)
     with tune.using(shape):
+        if (g.is_contiguous() and gp.is_contiguous() and gm.is_contiguous() and tuple(gp.shape) == (N, H, W)
+                and tuple(gm.shape) == (N, B, H // 2, W // 2)):
+            _C.dwtfuse_fuse_backward_batched_uniform(g, wavelet, gp, gm, ws)
+            return
         for i0 in range(0, N, _C.MAX_SCENES):
             scenes = [_C.make_grad_scene(g[i], wavelet, gp[i], gm[i])
                       for i in range(i0, min(N, i0 + _C.MAX_SCENES))]

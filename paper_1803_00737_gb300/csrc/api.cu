@@ -565,6 +565,64 @@ int dwtfuse_fuse_batched(const dwtfuse_scene *scenes, int n, void *workspace, si
     return cuda_status(launch_fuse_batched(t, queue, status, blocks_per_sm, static_cast<cudaStream_t>(stream)));
 }
 
+int dwtfuse_fuse_batched_uniform(const void *pan, const void *ms, int64_t n, int bands, int64_t H, int64_t W,
+                                 int wavelet, int in_dtype, float *out_f32, uint8_t *out_u8, void *workspace,
+                                 size_t ws_bytes, int rows_per_item_, int blocks_per_sm, void *stream) {
+    if (!pan || !ms || n < 1 || bands < 1) return DWTFUSE_EINVAL;
+    if (in_dtype != DWTFUSE_U8 && in_dtype != DWTFUSE_F32) return DWTFUSE_EINVAL;
+    int st = check_shape(H, W, wavelet);  // before any address is formed from the sizes
+    if (st != DWTFUSE_OK) return st;
+    if (bands > kBatchMaxBands) return DWTFUSE_ESHAPE;
+    const int64_t es = in_dtype == DWTFUSE_F32 ? 4 : 1, px = H * W, mpx = px / 4;
+    static thread_local dwtfuse_scene d[DWTFUSE_MAX_SCENES];
+    for (int64_t i0 = 0; i0 < n; i0 += DWTFUSE_MAX_SCENES) {
+        const int m = (int)(n - i0 < DWTFUSE_MAX_SCENES ? n - i0 : DWTFUSE_MAX_SCENES);
+        for (int k = 0; k < m; ++k) {
+            const int64_t i = i0 + k;
+            d[k].pan = static_cast<const char *>(pan) + i * px * es;
+            for (int b = 0; b < bands; ++b) d[k].ms[b] = static_cast<const char *>(ms) + (i * bands + b) * mpx * es;
+            d[k].out_f32 = out_f32 ? out_f32 + i * bands * px : nullptr;
+            d[k].out_u8 = out_u8 ? out_u8 + i * bands * px : nullptr;
+            d[k].H = H;
+            d[k].W = W;
+            d[k].bands = bands;
+            d[k].wavelet = wavelet;
+            d[k].in_dtype = in_dtype;
+            d[k].reserved = 0;
+        }
+        st = dwtfuse_fuse_batched(d, m, workspace, ws_bytes, rows_per_item_, blocks_per_sm, stream);
+        if (st != DWTFUSE_OK) return st;
+    }
+    return DWTFUSE_OK;
+}
+
+int dwtfuse_fuse_backward_batched_uniform(const float *grad_out, int64_t n, int bands, int64_t H, int64_t W,
+                                          int wavelet, float *grad_pan, float *grad_ms, void *workspace,
+                                          size_t ws_bytes, void *stream) {
+    if (!grad_out || !grad_pan || !grad_ms || n < 1 || bands < 1) return DWTFUSE_EINVAL;
+    int st = check_shape(H, W, wavelet);
+    if (st != DWTFUSE_OK) return st;
+    if (bands > kMaxBands) return DWTFUSE_ESHAPE;
+    const int64_t px = H * W, mpx = px / 4;
+    static thread_local dwtfuse_grad_scene d[DWTFUSE_MAX_SCENES];
+    for (int64_t i0 = 0; i0 < n; i0 += DWTFUSE_MAX_SCENES) {
+        const int m = (int)(n - i0 < DWTFUSE_MAX_SCENES ? n - i0 : DWTFUSE_MAX_SCENES);
+        for (int k = 0; k < m; ++k) {
+            const int64_t i = i0 + k;
+            d[k].grad_out = grad_out + i * bands * px;
+            d[k].grad_pan = grad_pan + i * px;
+            for (int b = 0; b < bands; ++b) d[k].grad_ms[b] = grad_ms + (i * bands + b) * mpx;
+            d[k].H = H;
+            d[k].W = W;
+            d[k].bands = bands;
+            d[k].wavelet = wavelet;
+        }
+        st = dwtfuse_fuse_backward_batched(d, m, workspace, ws_bytes, stream);
+        if (st != DWTFUSE_OK) return st;
+    }
+    return DWTFUSE_OK;
+}
+
 int dwtfuse_get_last_device_status(const void *workspace, void *stream) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (!workspace) return noalloc_device_status(s);  // the no-alloc call's static array

@@ -19,6 +19,7 @@ missing or corrupt cache is rebuilt.
 """
 from __future__ import annotations
 
+import functools
 import json
 import math
 import os
@@ -111,11 +112,17 @@ def device_key(name: str, sms: int, cc: tuple[int, int], driver: int) -> str:
     return f"{name}|sm{sms}|cc{cc[0]}{cc[1]}|drv{driver}"
 
 
-def current_device_key() -> str:
+@functools.lru_cache(maxsize=64)
+def _device_key(index: int) -> str:
     import torch
-    p = torch.cuda.get_device_properties(torch.cuda.current_device())
+    p = torch.cuda.get_device_properties(index)
     drv = torch.cuda.driver_version() if hasattr(torch.cuda, "driver_version") else 0
     return device_key(p.name, p.multi_processor_count, (p.major, p.minor), int(drv or 0))
+
+
+def current_device_key() -> str:
+    import torch
+    return _device_key(torch.cuda.current_device())
 
 
 def batched_class(specs: Iterable[tuple[int, int, int, int]]) -> str:
@@ -159,10 +166,23 @@ def _entry_shape(e) -> LaunchShape | None:
         return None
 
 
+_seen: tuple = (None, {})  # (path and file state, its entries) of the cache file last read by cached()
+
+
 def cached(key: str, path: str | None = None) -> LaunchShape | None:
-    """The cached shape for a key, or None (no tuning)."""
-    with _lock:
-        e = load_cache(path)["entries"].get(key)
+    """The cached shape for a key, or None (no tuning).  The file is read again
+    when it has changed (save_cache replaces it: another inode)."""
+    global _seen
+    path = path or cache_path()
+    try:
+        st = os.stat(path)
+    except OSError:
+        return None
+    state = (path, st.st_ino, st.st_mtime_ns, st.st_size)
+    seen = _seen
+    if seen[0] != state:
+        seen = _seen = (state, load_cache(path)["entries"])
+    e = seen[1].get(key)
     return _entry_shape(e) if e is not None else None
 
 
