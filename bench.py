@@ -94,6 +94,9 @@ KNOWN_TRAFFIC: dict[str, float] = {
     # row heights per launch, scalar synthesis where registers are short:
     # read 709,261,440 + write 8,006,737,536 (mean of 2 launches)
     "4ac0e872cfb0": 8715998976.0,
+    # fixed-point partial rows:
+    # read 706,983,424 + write 8,004,121,216 (mean of 2 launches)
+    "aac3151ae716": 8711104640.0,
 }
 KERNEL_SOURCES = ("fuse_tile.cuh", "fuse_metrics.cu", "metric_q.cuh", "tmem.cuh")
 

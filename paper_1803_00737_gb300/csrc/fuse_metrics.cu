@@ -300,24 +300,26 @@ fuse_metrics_kernel(const __grid_constant__ SceneArgs s, double *partial, int st
     tmem_fence_after();
     if (warp == 0) tmem_dealloc(*tmem_base, L::kTmemCols);
 
-    // One partial row per CTA, in the layout of the PAN-resolution pass:
-    // Q sums of the P pairs, then the NB squared-error sums (fixed order).
-    double *outp = partial + (int64_t)blockIdx.x * stride;
-    for (int k = threadIdx.x; k < L::P + NB; k += L::kThreads) {
-        double acc = 0.0;
-        for (int w = 0; w < L::kWarps; ++w) {
-            const unsigned char *wbw = fm_smem + w * L::kWarpBytes;
-            if (k < L::P) {
-                const float *qw = reinterpret_cast<const float *>(wbw) + L::kTile + L::kRep + L::kGsum;
-                for (int g = 0; g < 4; ++g) acc += (double)qw[g * L::P + k];
-            } else {
-                const long long *sw = reinterpret_cast<const long long *>(wbw + L::kWords * 4);
-                long long t = 0;
-                for (int l = 0; l < 32; ++l) t += sw[(k - L::P) * 32 + l];
-                acc += (double)t;
+    // One partial row per CTA, in the layout of the PAN-resolution pass: Q sums
+    // of the P pairs, then the NB squared-error sums.
+    long long *outp = reinterpret_cast<long long *>(partial) + (int64_t)blockIdx.x * stride;
+    // One warp per entry at a time, as integers (fixed-point Q sums, exact
+    // squared errors: FP64 adds run at 2 lanes a clock).
+    for (int k = warp; k < L::P + NB; k += L::kWarps) {
+        long long t = 0;
+        if (k < L::P) {
+            for (int i = lane; i < 4 * L::kWarps; i += 32) {
+                const float *qw = reinterpret_cast<const float *>(fm_smem + (i >> 2) * L::kWarpBytes) + L::kTile +
+                                  L::kRep + L::kGsum;
+                t += __float2ll_rn(qw[(i & 3) * L::P + k] * (float)(1ll << kQFracBits));
             }
+        } else {
+            for (int w = 0; w < L::kWarps; ++w)
+                t += reinterpret_cast<const long long *>(fm_smem + w * L::kWarpBytes +
+                                                         L::kWords * 4)[(k - L::P) * 32 + lane];
         }
-        outp[k] = acc;
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) outp[k] = t;
     }
 }
 

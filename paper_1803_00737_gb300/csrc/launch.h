@@ -33,6 +33,7 @@ static_assert(sizeof(BatchTable) + 16 <= 32764, "batched scene table exceeds the
 // kMetricStride for the PAN-resolution pass and as many for the MS pass.
 constexpr int kMetricMaxCtas = 1024;
 constexpr int kMetricStride = 64;    // >= pairs + bands for 8 bands (36 + 8)
+constexpr int kQFracBits = 40;       // fixed-point Q sums of the 8-bit passes' partial rows
 constexpr int kMetricMaxBands = 8;
 constexpr int kMetricWindow = 32;
 constexpr size_t kMetricWorkspaceBytes = sizeof(double) * (8 + 2 * (size_t)kMetricMaxCtas * kMetricStride);

@@ -308,15 +308,6 @@ __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)_
 __device__ __forceinline__ void mbar_init(uint64_t *bar) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, unsigned bytes) {
-    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.release.cta.shared::cta.b64 st, [%0];\n}\n" ::"r"(
-                     smem_u32(bar))
-                 : "memory");
-}
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, unsigned parity) {
     unsigned ok;
     asm volatile(
@@ -349,54 +340,108 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, unsigned parity) {
 static __device__ __noinline__ void stage_bytes(unsigned char *dst, uintptr_t c0, uintptr_t from, uintptr_t to) {
     for (uintptr_t p = from; p < to; ++p) dst[p - c0] = __ldg(reinterpret_cast<const uint8_t *>(p));
 }
-__device__ __forceinline__ void stage_row(unsigned char *dst, const uint8_t *a0, int len, const uint8_t *lo,
-                                          const uint8_t *hi, uint64_t *bar) {
-    const uintptr_t ua = reinterpret_cast<uintptr_t>(a0), c0 = ua & ~(uintptr_t)15, ue = ua + (uintptr_t)len;
-    const uintptr_t ulo = reinterpret_cast<uintptr_t>(lo), uhi = reinterpret_cast<uintptr_t>(hi);
-    uintptr_t bs = c0, be = (ue + 15) & ~(uintptr_t)15;
-    if (bs < ulo) bs = (ulo + 15) & ~(uintptr_t)15;
-    if (be > uhi) be = uhi & ~(uintptr_t)15;
-    if (be > bs) {
-        const unsigned n = (unsigned)(be - bs);
-        mbar_expect_tx(bar, n);
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-                         smem_u32(dst + (bs - c0))),
-                     "l"(reinterpret_cast<const void *>(bs)), "r"(n), "r"(smem_u32(bar))
-                     : "memory");
-        if (ua < bs) stage_bytes(dst, c0, ua, bs);
-        if (be < ue) stage_bytes(dst, c0, be, ue);
-    } else {
-        stage_bytes(dst, c0, ua, ue);
+// The in-plane chunks [bs, be) that cover row bytes [a0, a0 + len) of the plane
+// [lo, hi); none when be <= bs.
+struct RowSpan {
+    uintptr_t ua = 0, ue = 0, c0 = 0, bs = 0, be = 0;
+    __device__ __forceinline__ RowSpan() {}
+    __device__ __forceinline__ RowSpan(const uint8_t *a0, int len, const uint8_t *lo, const uint8_t *hi) {
+        ua = reinterpret_cast<uintptr_t>(a0);
+        ue = ua + (uintptr_t)len;
+        c0 = ua & ~(uintptr_t)15;
+        const uintptr_t ulo = reinterpret_cast<uintptr_t>(lo), uhi = reinterpret_cast<uintptr_t>(hi);
+        bs = c0;
+        be = (ue + 15) & ~(uintptr_t)15;
+        if (bs < ulo) bs = (ulo + 15) & ~(uintptr_t)15;
+        if (be > uhi) be = uhi & ~(uintptr_t)15;
     }
+    __device__ __forceinline__ unsigned bytes() const { return be > bs ? (unsigned)(be - bs) : 0u; }
+};
+// The covering chunks of row bytes [a0, a0 + len), not clipped.
+__device__ __forceinline__ unsigned span_bytes(const uint8_t *a0, int len) {
+    return ((unsigned)(reinterpret_cast<uintptr_t>(a0) & 15) + (unsigned)len + 15u) & ~15u;
+}
+// Whether the covering chunks of rows a0, a0 + step, ... (n rows) all lie in
+// [lo, hi).
+__device__ __forceinline__ bool spans_inside(const uint8_t *a0, int64_t step, int n, int len, const uint8_t *lo,
+                                             const uint8_t *hi) {
+    const uintptr_t first = reinterpret_cast<uintptr_t>(a0) & ~(uintptr_t)15;
+    const uintptr_t last = (reinterpret_cast<uintptr_t>(a0 + (n - 1) * step + len) + 15) & ~(uintptr_t)15;
+    return first >= reinterpret_cast<uintptr_t>(lo) && last <= reinterpret_cast<uintptr_t>(hi);
+}
+__device__ __forceinline__ void copy_span(unsigned char *dst, const uint8_t *a0, unsigned bytes, uint64_t *bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                     smem_u32(dst)),
+                 "l"(reinterpret_cast<const void *>(reinterpret_cast<uintptr_t>(a0) & ~(uintptr_t)15)), "r"(bytes),
+                 "r"(smem_u32(bar))
+                 : "memory");
+}
+__device__ __forceinline__ void stage_row(unsigned char *dst, const RowSpan &r, uint64_t *bar) {
+    if (r.be > r.bs) {
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                         smem_u32(dst + (r.bs - r.c0))),
+                     "l"(reinterpret_cast<const void *>(r.bs)), "r"(r.bytes()), "r"(smem_u32(bar))
+                     : "memory");
+        if (r.ua < r.bs) stage_bytes(dst, r.c0, r.ua, r.bs);
+        if (r.be < r.ue) stage_bytes(dst, r.c0, r.be, r.ue);
+    } else if (r.ue > r.ua) {
+        stage_bytes(dst, r.c0, r.ua, r.ue);
+    }
+}
+
+// Row slots per warp of the MS-resolution pass: a CTA's slots are shared out
+// over its warps that have an item (items go round the CTAs, so a scene with
+// fewer items than warps leaves some without), up to kMaxStages each: a warp
+// then has more rows in flight (7480 x 8140 x 6: the pass 76 -> 69 us; the
+// PAN-resolution pass, whose CTAs are full from 20 Mpx on, keeps its two).
+constexpr int kMaxStages = 8;
+__device__ __forceinline__ int ring_stages(int64_t items, int warps, int stages) {
+    int64_t busy = (items - blockIdx.x + gridDim.x - 1) / gridDim.x;
+    if (busy < 1) busy = 1;
+    if (busy >= warps) return stages;
+    const int s = warps * stages / (int)busy;
+    return s < kMaxStages ? s : kMaxStages;
 }
 
 // Per-warp ring of row slots for the unaligned path: slot k's mbarrier
 // completes when every bulk copy of the row staged there has landed (the one
-// arrival is lane 0's, after all lanes have posted their byte counts).
-template <int S>
+// arrival is lane 0's, with the sum of all lanes' byte counts, before any copy
+// is issued).  FS: stages, 0 for a number given at run time.
+template <int FS>
 struct BulkRing {
     uint64_t *bar;
+    int S;
     unsigned phase = 0;  // bit k: parity of slot k's next phase
     int issue_slot = 0, wait_slot = 0, pending = 0;
-    __device__ __forceinline__ void init(uint64_t *bars, int lane) {
+    __device__ __forceinline__ void init(uint64_t *bars, int stages, int lane) {
         bar = bars;
+        S = FS ? FS : stages;
         if (lane == 0)
             for (int k = 0; k < S; ++k) mbar_init(bar + k);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         __syncwarp();
     }
-    // after this lane staged its plane's row into slot issue_slot
-    __device__ __forceinline__ void commit(int lane) {
+    // Starts a row: every lane's copy of `bytes` into slot issue_slot follows.
+    __device__ __forceinline__ void begin(unsigned bytes, int lane) {
+        const unsigned all = __reduce_add_sync(0xffffffffu, bytes);
+        if (lane == 0) {
+            asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(
+                             smem_u32(bar + issue_slot)),
+                         "r"(all)
+                         : "memory");
+        }
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar + issue_slot);
-        issue_slot = issue_slot + 1 == S ? 0 : issue_slot + 1;
+    }
+    // after this lane staged its plane's row into slot issue_slot
+    __device__ __forceinline__ void commit() {
+        issue_slot = issue_slot + 1 == (FS ? FS : S) ? 0 : issue_slot + 1;
         ++pending;
     }
     __device__ __forceinline__ bool wait() {
         const bool ok = mbar_wait_warp(bar + wait_slot, (phase >> wait_slot) & 1u);
         if (ok) {
             phase ^= 1u << wait_slot;
-            wait_slot = wait_slot + 1 == S ? 0 : wait_slot + 1;
+            wait_slot = wait_slot + 1 == (FS ? FS : S) ? 0 : wait_slot + 1;
             --pending;
         }
         __syncwarp();
@@ -407,11 +452,23 @@ struct BulkRing {
         while (pending > 0) {
             mbar_wait_warp(bar + wait_slot, (phase >> wait_slot) & 1u);
             phase ^= 1u << wait_slot;
-            wait_slot = wait_slot + 1 == S ? 0 : wait_slot + 1;
+            wait_slot = wait_slot + 1 == (FS ? FS : S) ? 0 : wait_slot + 1;
             --pending;
         }
     }
 };
+// cp.async.wait_group S - 1 for a run-time number of stages.
+__device__ __forceinline__ void cp_async_wait_stages(int S) {
+    switch (S) {
+        case 2: cp_async_wait<1>(); break;
+        case 3: cp_async_wait<2>(); break;
+        case 4: cp_async_wait<3>(); break;
+        case 5: cp_async_wait<4>(); break;
+        case 6: cp_async_wait<5>(); break;
+        case 7: cp_async_wait<6>(); break;
+        default: cp_async_wait<7>(); break;
+    }
+}
 
 // NW 32-bit words of a staged row starting at byte offset off (one offset per
 // image row, the same for every lane, so the branches are uniform).  Lanes
@@ -502,6 +559,38 @@ struct FastPan {
     static constexpr int kSmem = kBarOffset + kFastWarps * kStages * 8;  // with the mbarriers (GEN)
 };
 
+// Partial rows of the 8-bit passes are int64: Q sums in units of 2^-kQFracBits,
+// squared errors and MS sums exact.  FP64 runs at 2 lanes a clock on an SM:
+// adding a CTA's 256 Q values per pair in FP64, and up to 456 rows of doubles
+// in the finalize, took about 10 and 18 us; as integers 1-2 and 5.
+__device__ __forceinline__ long long q_fixed(float q) { return __float2ll_rn(q * (float)(1ll << kQFracBits)); }
+
+// The CTA's partial row from the warps' Q slots (sq: [warps][windows][P]
+// floats) and sums (sum: [warps][NB] doubles, exact integers).  One warp per
+// pair at a time: its lanes add the slots (in a fixed order), then a butterfly.
+template <int P, int NB, int WARPS>
+__device__ __forceinline__ void write_partial(long long *out, const float *sq, const double *sum) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int k = warp; k < P; k += WARPS) {
+        long long a = 0;
+        for (int s = lane; s < WARPS * kWinPerStrip; s += 32) a += q_fixed(sq[s * P + k]);
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) out[k] = a;
+    }
+    if (threadIdx.x < NB) {
+        long long a = 0;
+        for (int w = 0; w < WARPS; ++w) a += __double2ll_rn(sum[w * NB + threadIdx.x]);
+        out[P + threadIdx.x] = a;
+    }
+}
+
+// The pass is bound by its instructions (ncu, 7480 x 8140 x 6: 62 % of issue
+// slots): items go round the CTAs (with 1.5 items a warp, CTAs of consecutive
+// items left half of the SMs idle in the second round: 188 -> 156 us), the row
+// copies post one byte count instead of one per plane, and skip the clipping
+// where no row of the item can leave its plane (832 -> 700 instructions a row).
+// The float order of a warp's Q sums is that of its items, as before.
+//
 // GEN = false: rows of every plane start on 16-byte boundaries (W % 16 == 0,
 // aligned planes): one cp.async chunk per lane and image, read back by the
 // same lane.  GEN = true: any width and alignment; lane p stages plane p's row
@@ -515,12 +604,11 @@ metrics_pan_u8_kernel(const __grid_constant__ MetricArgs a) {
     allow_dependents();
     using C = FastPan<NB, GEN>;
     constexpr int kFastWarps = C::kWarps;
-    constexpr int K = C::K, P = C::P, S = C::kStages, RB = C::kRowBytes;
+    constexpr int K = C::K, P = C::P, RB = C::kRowBytes, kSlots = kFastWarps * C::kStages;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned char *ring = smem + warp * S * RB;
-    float *sq = reinterpret_cast<float *>(smem + kFastWarps * S * RB) + warp * kWinPerStrip * P;
-    double *sse = reinterpret_cast<double *>(smem + kFastWarps * S * RB + kFastWarps * kWinPerStrip * P * 4);
+    float *sq = reinterpret_cast<float *>(smem + kSlots * RB) + warp * kWinPerStrip * P;
+    double *sse = reinterpret_cast<double *>(smem + kSlots * RB + kFastWarps * kWinPerStrip * P * 4);
     for (int k = lane; k < kWinPerStrip * P; k += 32) sq[k] = 0.f;
     double se_tot[NB];
 #pragma unroll
@@ -531,16 +619,19 @@ metrics_pan_u8_kernel(const __grid_constant__ MetricArgs a) {
     const int64_t sx_n = (W + kStrip - 1) / kStrip, sy_n = (H + kWin - 1) / kWin;
     const int64_t items = sx_n * sy_n;
     const int64_t nw = (int64_t)gridDim.x * kFastWarps;
+    constexpr int S = C::kStages;
+    unsigned char *ring = smem + warp * S * RB;
     // GEN: this lane's plane -- fused band `lane`, PAN (lane NB, when Q is
     // wanted), MS band lane - NB - 1 -- and where its rows go in a slot.
-    BulkRing<S> br;
+    BulkRing<C::kStages> br;
     const uint8_t *pl = nullptr;
     int64_t pl_n = 0;
     int kind = 0, dst_off = 0;  // kind 1: PAN-resolution row, 2: MS row
     bool err = false;
     bool stall = GEN && a.wait_test && blockIdx.x == 0 && warp == 0;  // test hook, first slot only
-    if (GEN) {
-        br.init(reinterpret_cast<uint64_t *>(smem + C::kBarOffset) + warp * S, lane);
+    const bool has_item = (int64_t)warp * gridDim.x + blockIdx.x < items;
+    if (GEN && has_item) {
+        br.init(reinterpret_cast<uint64_t *>(smem + C::kBarOffset) + warp * S, S, lane);
         if (lane < NB) {
             pl = F + (int64_t)lane * HW; pl_n = HW; kind = 1; dst_off = lane * kImgRow;
         } else if (lane == NB) {
@@ -550,7 +641,7 @@ metrics_pan_u8_kernel(const __grid_constant__ MetricArgs a) {
             pl = static_cast<const uint8_t *>(a.ms[b]); pl_n = H2 * W2; kind = 2; dst_off = K * kImgRow + b * kMsRow;
         }
     }
-    for (int64_t it = (int64_t)blockIdx.x * kFastWarps + warp; it < items; it += nw) {
+    for (int64_t it = (int64_t)warp * gridDim.x + blockIdx.x; it < items; it += nw) {  // items round the CTAs first
         const int64_t x0 = (it % sx_n) * kStrip;
         const int64_t x = x0 + kLanePx * lane;
         const int64_t y0 = (it / sx_n) * kWin;
@@ -560,27 +651,41 @@ metrics_pan_u8_kernel(const __grid_constant__ MetricArgs a) {
         const bool full = a.want_q && (y0 + kWin <= H) && (xwin + kWin <= W);
         const int nrows = (int)min((int64_t)kWin, H - y0);
         const int span = (int)min((int64_t)kStrip, W - x0);
-        // Row r of this strip into the next ring slot (r % S on the aligned path).
+        const int len = kind == 2 ? span / 2 : span;
+        const uint8_t *next = nullptr;  // GEN: the lane's plane row to stage next
+        bool inside = true;
+        if (GEN) {
+            if (kind) {
+                next = kind == 1 ? pl + y0 * W + x0 : pl + (y0 >> 1) * W2 + (x0 >> 1);
+                inside = spans_inside(next, kind == 1 ? W : W2, kind == 1 ? nrows : (nrows + 1) / 2, len, pl, pl + pl_n);
+            }
+            inside = __all_sync(0xffffffffu, inside);
+        }
+        // Row r of this strip into the next ring slot (`fill` on the aligned path).
+        int fill = 0, take = 0;
         auto issue = [&](int r) {
             if (GEN) {
                 if (r < nrows) {
                     unsigned char *slot = ring + br.issue_slot * RB;
-                    const int64_t y = y0 + r;
-                    if (kind == 1)
-                        stage_row(slot + dst_off, pl + y * W + x0, span, pl, pl + pl_n, br.bar + br.issue_slot);
-                    else if (kind == 2)
-                        stage_row(slot + dst_off, pl + (y >> 1) * W2 + (x0 >> 1), span / 2, pl, pl + pl_n,
-                                  br.bar + br.issue_slot);
-                    if (stall) {
-                        if (lane == 0) mbar_expect_tx(br.bar + br.issue_slot, 16u);
-                        stall = false;
+                    const unsigned extra = stall && lane == 0 ? 16u : 0u;  // (test hook: bytes that no copy delivers)
+                    stall = false;
+                    if (inside) {  // no chunk leaves its plane: nothing to clip
+                        const unsigned n = kind ? span_bytes(next, len) : 0u;
+                        br.begin(n + extra, lane);
+                        if (n) copy_span(slot + dst_off, next, n, br.bar + br.issue_slot);
+                    } else {
+                        RowSpan rs;
+                        if (kind) rs = RowSpan(next, len, pl, pl + pl_n);
+                        br.begin(rs.bytes() + extra, lane);
+                        stage_row(slot + dst_off, rs, br.bar + br.issue_slot);
                     }
-                    br.commit(lane);
+                    next += kind == 1 ? W : ((r & 1) ? W2 : 0);  // an MS row serves two image rows
+                    br.commit();
                 }
                 return;
             }
             if (r < nrows) {
-                unsigned char *slot = ring + (r % S) * RB;
+                unsigned char *slot = ring + fill * RB;
                 const int64_t y = y0 + r;
                 if (act) {
 #pragma unroll
@@ -594,8 +699,8 @@ metrics_pan_u8_kernel(const __grid_constant__ MetricArgs a) {
                 }
             }
             cp_async_commit();
+            fill = fill + 1 == S ? 0 : fill + 1;
         };
-#pragma unroll
         for (int r = 0; r < S - 1; ++r) issue(r);
         int s1[K], s2[K], sxy[P], se[NB];
 #pragma unroll
@@ -622,8 +727,9 @@ metrics_pan_u8_kernel(const __grid_constant__ MetricArgs a) {
                 my_o = (int)(((unsigned)reinterpret_cast<uintptr_t>(pl) + rowbase) & 15u);
             } else {
                 issue(r + S - 1);
-                cp_async_wait<S - 1>();
-                slot = ring + (r % S) * RB;
+                cp_async_wait_stages(S);
+                slot = ring + take * RB;
+                take = take + 1 == S ? 0 : take + 1;
             }
             int o_f[NB], o_m[NB], o_p = 0;
             if (GEN) {
@@ -737,20 +843,10 @@ metrics_pan_u8_kernel(const __grid_constant__ MetricArgs a) {
         if (lane == 0) sse[warp * NB + b] = v;
     }
     const int any_err = __syncthreads_or(err);
-    const float *sq0 = reinterpret_cast<const float *>(smem + kFastWarps * S * RB);
-    double *out = a.partial + (int64_t)blockIdx.x * a.stride;
-    if (GEN && threadIdx.x == 0) out[P + NB] = any_err ? 1.0 : 0.0;
-    for (int k = threadIdx.x; k < P + NB; k += kFastWarps * 32) {
-        double acc = 0.0;
-        for (int w = 0; w < kFastWarps; ++w) {
-            if (k < P) {
-                for (int s = 0; s < kWinPerStrip; ++s) acc += (double)sq0[(w * kWinPerStrip + s) * P + k];
-            } else {
-                acc += sse[w * NB + k - P];
-            }
-        }
-        out[k] = acc;
-    }
+    const float *sq0 = reinterpret_cast<const float *>(smem + kSlots * RB);
+    long long *out = reinterpret_cast<long long *>(a.partial) + (int64_t)blockIdx.x * a.stride;
+    if (GEN && threadIdx.x == 0) out[P + NB] = any_err ? 1 : 0;
+    write_partial<P, NB, kFastWarps>(out, sq0, sse);
 }
 
 // MS-resolution pass: up to 6 bands, 8-warp CTAs, two per SM.  Against
@@ -794,12 +890,11 @@ __global__ void __launch_bounds__(FastMs<NB, GEN>::kWarps * 32, FastMs<NB, GEN>:
 metrics_ms_u8_kernel(const __grid_constant__ MetricArgs a) {
     using C = FastMs<NB, GEN>;
     constexpr int kFastWarps = C::kWarps;
-    constexpr int K = C::K, P = C::P, S = C::kStages, RB = C::kRowBytes, PR = C::kPanRow;
+    constexpr int K = C::K, P = C::P, RB = C::kRowBytes, PR = C::kPanRow, kSlots = kFastWarps * C::kStages;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned char *ring = smem + warp * S * RB;
-    float *sq = reinterpret_cast<float *>(smem + kFastWarps * S * RB) + warp * kWinPerStrip * P;
-    double *ssum = reinterpret_cast<double *>(smem + kFastWarps * S * RB + kFastWarps * kWinPerStrip * P * 4);
+    float *sq = reinterpret_cast<float *>(smem + kSlots * RB) + warp * kWinPerStrip * P;
+    double *ssum = reinterpret_cast<double *>(smem + kSlots * RB + kFastWarps * kWinPerStrip * P * 4);
     for (int k = lane; k < kWinPerStrip * P; k += 32) sq[k] = 0.f;
     double sum_tot[NB];
 #pragma unroll
@@ -809,13 +904,16 @@ metrics_ms_u8_kernel(const __grid_constant__ MetricArgs a) {
     const int64_t sx_n = (W2 + kStrip - 1) / kStrip, sy_n = (H2 + kWin - 1) / kWin;
     const int64_t items = sx_n * sy_n;
     const int64_t nw = (int64_t)gridDim.x * kFastWarps;
-    BulkRing<S> br;
+    const int S = ring_stages(items, kFastWarps, C::kStages);
+    unsigned char *ring = smem + warp * S * RB;  // (used by warps with an item)
+    BulkRing<0> br;
     const uint8_t *pl = nullptr;
     int64_t pl_n = 0;
     int kind = 0, dst_off = 0;  // kind 1: MS row, 2: PAN row 2i + (lane - NB)
     bool err = false;
-    if (GEN) {
-        br.init(reinterpret_cast<uint64_t *>(smem + C::kBarOffset) + warp * S, lane);
+    const bool has_item = (int64_t)warp * gridDim.x + blockIdx.x < items;
+    if (GEN && has_item) {
+        br.init(reinterpret_cast<uint64_t *>(smem + C::kBarOffset) + warp * S, S, lane);
         if (lane < NB) {
             pl = static_cast<const uint8_t *>(a.ms[lane]); pl_n = H2 * W2; kind = 1; dst_off = lane * kImgRow;
         } else if (lane < NB + 2) {
@@ -833,22 +931,37 @@ metrics_ms_u8_kernel(const __grid_constant__ MetricArgs a) {
         const bool any_full = __any_sync(0xffffffffu, full);
         const int nrows = (int)min((int64_t)kWin, H2 - i0);
         const int span = (int)min((int64_t)kStrip, W2 - j0);
+        const int len = kind == 2 ? 2 * span : span;
+        const uint8_t *next = nullptr;  // GEN: the lane's plane row to stage next (none: no row wanted)
+        bool inside = true;
+        if (GEN) {
+            if (kind == 1) next = pl + i0 * W2 + j0;
+            if (kind == 2 && any_full) next = pl + (2 * i0 + (lane - NB)) * W + 2 * j0;
+            if (next) inside = spans_inside(next, kind == 1 ? W2 : 2 * W, nrows, len, pl, pl + pl_n);
+            inside = __all_sync(0xffffffffu, inside);
+        }
+        int fill = 0, take = 0;
         auto issue = [&](int r) {
             if (GEN) {
                 if (r < nrows) {
                     unsigned char *slot = ring + br.issue_slot * RB;
-                    const int64_t i = i0 + r;
-                    if (kind == 1)
-                        stage_row(slot + dst_off, pl + i * W2 + j0, span, pl, pl + pl_n, br.bar + br.issue_slot);
-                    else if (kind == 2 && any_full)
-                        stage_row(slot + dst_off, pl + (2 * i + (lane - NB)) * W + 2 * j0, 2 * span, pl, pl + pl_n,
-                                  br.bar + br.issue_slot);
-                    br.commit(lane);
+                    if (inside) {  // no chunk leaves its plane: nothing to clip
+                        const unsigned n = next ? span_bytes(next, len) : 0u;
+                        br.begin(n, lane);
+                        if (n) copy_span(slot + dst_off, next, n, br.bar + br.issue_slot);
+                    } else {
+                        RowSpan rs;
+                        if (next) rs = RowSpan(next, len, pl, pl + pl_n);
+                        br.begin(rs.bytes(), lane);
+                        stage_row(slot + dst_off, rs, br.bar + br.issue_slot);
+                    }
+                    if (next) next += kind == 1 ? W2 : 2 * W;
+                    br.commit();
                 }
                 return;
             }
             if (r < nrows) {
-                unsigned char *slot = ring + (r % S) * RB;
+                unsigned char *slot = ring + fill * RB;
                 const int64_t i = i0 + r;
                 if (act) {
 #pragma unroll
@@ -864,8 +977,8 @@ metrics_ms_u8_kernel(const __grid_constant__ MetricArgs a) {
                 }
             }
             cp_async_commit();
+            fill = fill + 1 == S ? 0 : fill + 1;
         };
-#pragma unroll
         for (int r = 0; r < S - 1; ++r) issue(r);
         int s1[K], s2[K], sxy[P], sm[NB];
 #pragma unroll
@@ -892,8 +1005,9 @@ metrics_ms_u8_kernel(const __grid_constant__ MetricArgs a) {
                 my_o = (int)(((unsigned)reinterpret_cast<uintptr_t>(pl) + rowbase) & 15u);
             } else {
                 issue(r + S - 1);
-                cp_async_wait<S - 1>();
-                slot = ring + (r % S) * RB;
+                cp_async_wait_stages(S);
+                slot = ring + take * RB;
+                take = take + 1 == S ? 0 : take + 1;
             }
             int o_m[NB], o_p0 = 0, o_p1 = 0;
             if (GEN) {
@@ -1012,20 +1126,10 @@ metrics_ms_u8_kernel(const __grid_constant__ MetricArgs a) {
         if (lane == 0) ssum[warp * NB + b] = v;
     }
     const int any_err = __syncthreads_or(err);
-    const float *sq0 = reinterpret_cast<const float *>(smem + kFastWarps * S * RB);
-    double *out = a.partial + (int64_t)blockIdx.x * a.stride;
-    if (GEN && threadIdx.x == 0) out[P + NB] = any_err ? 1.0 : 0.0;
-    for (int k = threadIdx.x; k < P + NB; k += kFastWarps * 32) {
-        double acc = 0.0;
-        for (int w = 0; w < kFastWarps; ++w) {
-            if (k < P) {
-                for (int s = 0; s < kWinPerStrip; ++s) acc += (double)sq0[(w * kWinPerStrip + s) * P + k];
-            } else {
-                acc += ssum[w * NB + k - P];
-            }
-        }
-        out[k] = acc;
-    }
+    const float *sq0 = reinterpret_cast<const float *>(smem + kSlots * RB);
+    long long *out = reinterpret_cast<long long *>(a.partial) + (int64_t)blockIdx.x * a.stride;
+    if (GEN && threadIdx.x == 0) out[P + NB] = any_err ? 1 : 0;
+    write_partial<P, NB, kFastWarps>(out, sq0, ssum);
     wait_primary();  // a programmatic dependent completes only after its primary grid
 }
 
@@ -1126,31 +1230,58 @@ metrics_ms_kernel(const __grid_constant__ MetricArgs a) {
 // D_lambda, D_s (QNR terms NaN when not requested or when no full window
 // exists at either resolution; all four NaN when a pass flagged in
 // `status_mask` (bit 0 PAN-resolution, bit 1 MS) reported a wait that gave up
-// in entry P + nb of a partial row).  Each warp reduces one column of partials:
-// lanes stride over the CTAs, then a xor butterfly (a fixed order, so the
-// result is the same on every run).  The lane loop is unrolled so that its
-// loads are in flight together: the partials sit in L2 and each round trip
-// is a few hundred cycles.
-constexpr int kFinalizeThreads = 1024;
+// in entry P + nb of a partial row), to `out` and, where given, `result`.
+// Thread (g, k) adds column k of rows g, g + 16, ...: 64 threads read a row's
+// 512 bytes together; then 16 sums per column (a fixed order, so the result is
+// the same on every run).  fixed_mask: passes whose rows are int64.
+constexpr int kFinalizeGroups = 16;
+constexpr int kFinalizeThreads = kFinalizeGroups * kMetricStride;
+template <typename S>
+__device__ __forceinline__ S column_sum(const double *part, int ctas, int g, int k) {
+    const S *p = reinterpret_cast<const S *>(part) + k;
+    S a = 0;
+#pragma unroll 8
+    for (int c = g; c < ctas; c += kFinalizeGroups) a += p[(int64_t)c * kMetricStride];
+    return a;
+}
 __global__ void __launch_bounds__(kFinalizeThreads)
 metrics_finalize_kernel(const double *pan_part, const double *ms_part, int ctas_pan, const int *ctas_pan_dev,
-                        int ctas_ms, int stride, int nb, int want_q, int64_t H, int64_t W, int64_t nwin_pan,
-                        int64_t nwin_ms, int status_mask, double *out) {
+                        int ctas_ms, int nb, int want_q, int64_t H, int64_t W, int64_t nwin_pan,
+                        int64_t nwin_ms, int status_mask, int fixed_mask, double *out, double *result) {
+    wait_primary();  // programmatic dependent of the MS-resolution pass
     if (ctas_pan_dev) ctas_pan = *ctas_pan_dev;
-    __shared__ double tot_pan[64 + kMaxBands];
-    __shared__ double tot_ms[64 + kMaxBands];
+    __shared__ double part[2][kFinalizeGroups][kMetricStride];  // (int64 bits of a fixed-point pass)
+    __shared__ double tot_pan[kMetricStride];
+    __shared__ double tot_ms[kMetricStride];
     const int P = nb * (nb - 1) / 2 + nb;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (int k = warp; k < 2 * (P + nb + 1); k += nwarps) {
-        const bool ms = k >= P + nb + 1;
-        const int kk = ms ? k - (P + nb + 1) : k;
-        const double *part = ms ? ms_part : pan_part;
-        const int ctas = (kk < P + nb || ((status_mask >> (ms ? 1 : 0)) & 1)) ? (ms ? ctas_ms : ctas_pan) : 0;
-        double a = 0.0;
-#pragma unroll 8
-        for (int c = lane; c < ctas; c += 32) a += part[(int64_t)c * stride + kk];
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (lane == 0) (ms ? tot_ms : tot_pan)[kk] = a;
+    const int lane = threadIdx.x & 31;
+    {
+        const int g = threadIdx.x / kMetricStride, k = threadIdx.x % kMetricStride;
+#pragma unroll
+        for (int ms = 0; ms < 2; ++ms) {
+            const bool used = k < P + nb || (k == P + nb && ((status_mask >> ms) & 1));
+            const int ctas = used ? (ms ? ctas_ms : ctas_pan) : 0;
+            const double *src = ms ? ms_part : pan_part;
+            if ((fixed_mask >> ms) & 1)
+                part[ms][g][k] = __longlong_as_double(column_sum<long long>(src, ctas, g, k));
+            else
+                part[ms][g][k] = column_sum<double>(src, ctas, g, k);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * kMetricStride) {
+        const int ms = threadIdx.x / kMetricStride, k = threadIdx.x % kMetricStride;
+        double t;
+        if ((fixed_mask >> ms) & 1) {
+            long long a = 0;
+#pragma unroll
+            for (int g = 0; g < kFinalizeGroups; ++g) a += __double_as_longlong(part[ms][g][k]);
+            t = k < P ? (double)a * (1.0 / (double)(1ll << kQFracBits)) : (double)a;
+        } else {
+            t = 0.0;
+            for (int g = 0; g < kFinalizeGroups; ++g) t += part[ms][g][k];
+        }
+        (ms ? tot_ms : tot_pan)[k] = t;
     }
     __syncthreads();
     if (threadIdx.x >= 32) return;
@@ -1177,23 +1308,25 @@ metrics_finalize_kernel(const double *pan_part, const double *ms_part, int ctas_
         ds += __shfl_xor_sync(0xffffffffu, ds, o);
     }
     if (lane != 0) return;
-    int *status = reinterpret_cast<int *>(out + kMetricStatusSlot);
-    if (tot_pan[P + nb] + tot_ms[P + nb] > 0.0) {
-        out[0] = out[1] = out[2] = out[3] = __longlong_as_double(0x7ff8000000000000ll);
-        *status = DWTFUSE_ETIMEOUT;
-        return;
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    double r[4] = {nan, nan, nan, nan};
+    int status = DWTFUSE_ETIMEOUT;
+    if (!(tot_pan[P + nb] + tot_ms[P + nb] > 0.0)) {
+        status = DWTFUSE_OK;
+        r[0] = 100.0 * 0.5 * sqrt(e / nb);
+        if (q_ok) {
+            dl = nb > 1 ? 2.0 * dl / (nb * (nb - 1)) : 0.0;
+            ds /= nb;
+            r[1] = (1.0 - dl) * (1.0 - ds);
+            r[2] = dl;
+            r[3] = ds;
+        }
     }
-    *status = DWTFUSE_OK;
-    out[0] = 100.0 * 0.5 * sqrt(e / nb);
-    if (!q_ok) {
-        out[1] = out[2] = out[3] = __longlong_as_double(0x7ff8000000000000ll);
-        return;
+    *reinterpret_cast<int *>(out + kMetricStatusSlot) = status;
+    for (int k = 0; k < 4; ++k) {
+        out[k] = r[k];
+        if (result) result[k] = r[k];
     }
-    dl = nb > 1 ? 2.0 * dl / (nb * (nb - 1)) : 0.0;
-    ds /= nb;
-    out[1] = (1.0 - dl) * (1.0 - ds);
-    out[2] = dl;
-    out[3] = ds;
 }
 
 template <typename TF, typename TI, int NB>
@@ -1381,14 +1514,25 @@ cudaError_t launch_metrics(const MetricLaunch &m, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     const int64_t nwp = (m.H / kWin) * (m.W / kWin), nwm = (m.H / 2 / kWin) * (m.W / 2 / kWin);
     const int *gp_dev = m.pan_done ? reinterpret_cast<const int *>(m.workspace + kMetricPanCtasSlot) : nullptr;
-    metrics_finalize_kernel<<<1, kFinalizeThreads, 0, stream>>>(pan_part, ms_part, gp, gp_dev, gm, kMetricStride,
-                                                                m.bands, m.want_q, m.H, m.W, nwp, nwm, status_mask,
-                                                                out);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (m.result && m.result != out)
-        e = cudaMemcpyAsync(m.result, out, 4 * sizeof(double), cudaMemcpyDeviceToDevice, stream);
-    return e;
+    const int fixed_mask = (m.pan_done || fast ? 1 : 0) | (m.in_f32 ? 0 : 2);
+    double *result = m.result != out ? m.result : nullptr;
+    const double *pp = pan_part, *mp = ms_part;
+    int nb = m.bands, want_q = m.want_q;
+    int64_t H = m.H, W = m.W, nw_pan = nwp, nw_ms = nwm;
+    void *args3[] = {&pp, &mp, &gp, &gp_dev, &gm, &nb, &want_q, &H, &W, &nw_pan, &nw_ms, &status_mask,
+                     const_cast<int *>(&fixed_mask), &out, &result};
+    // Programmatic dependent of the MS pass: its launch overlaps that pass's
+    // end (it waits for the grid before it reads anything).
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1);
+    cfg.blockDim = dim3(kFinalizeThreads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(&metrics_finalize_kernel), args3);
 }
 
 }  // namespace dwtfuse
