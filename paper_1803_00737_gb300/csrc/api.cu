@@ -331,6 +331,7 @@ int dwtfuse_idwt2(const float *coeffs, int64_t H, int64_t W, int wavelet, float 
     d.wavelet = wavelet;
     d.inverse = 1;
     d.a4 = (W % 4 == 0) && (!out_f32 || aligned(out_f32, 16)) && (!out_u8 || aligned(out_u8, 4));
+    d.pairs = (W % 4 == 0) && aligned(coeffs, 8);
     d.rows = rows_per_item();
     return cuda_status(launch_dwt2(d, static_cast<cudaStream_t>(stream)));
 }

@@ -54,28 +54,17 @@ __device__ __forceinline__ void store_pair(float *p, bool pair, bool two, float 
     }
 }
 
-// Row analysis of one image row at coefficient columns n, n+1 (pixels x..x+5 = v[2..7]).
-__device__ __forceinline__ void d4_row_ad(const float *v, float *ra, float *rd) {
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const float *s = v + 2 + 2 * j;
-        ra[j] = fmaf(kH3, s[3], fmaf(kH2, s[2], fmaf(kH1, s[1], kH0 * s[0])));
-        rd[j] = fmaf(kG3, s[3], fmaf(kG2, s[2], fmaf(kG1, s[1], kG0 * s[0])));
-    }
-}
-
-// Raw uint8 words of one image row for a lane's D4 taps (pixels x-2..x+5,
-// periodic): the pair at x-2, the 4 pixels at x (one word on the vector path,
-// else two pairs), the pair at x+4.
-struct Raw8 {
-    uint32_t l, m0, m1, r;
+// Raw uint8 words of one image row for a lane's D4 taps (pixels x..x+5,
+// periodic): the 4 pixels at x (one word on the vector path, else two pairs),
+// the pair at x+4.
+struct Raw6 {
+    uint32_t m0, m1, r;
 };
 
 template <typename T>
-__device__ __forceinline__ Raw8 load_raw8(const T *row, const LaneCols &c, bool a4) {
+__device__ __forceinline__ Raw6 load_raw6(const T *row, const LaneCols &c, bool a4) {
     const uint8_t *p = reinterpret_cast<const uint8_t *>(row);
-    Raw8 w;
-    w.l = __ldg(reinterpret_cast<const unsigned short *>(p + c.cm));
+    Raw6 w;
     if (a4) {
         w.m0 = __ldg(reinterpret_cast<const unsigned int *>(p + c.x));
         w.m1 = 0;
@@ -87,16 +76,28 @@ __device__ __forceinline__ Raw8 load_raw8(const T *row, const LaneCols &c, bool 
     return w;
 }
 
-__device__ __forceinline__ void unpack_raw8(const Raw8 &w, bool a4, float *v) {
-    v[0] = byte_f(w.l, 0);
-    v[1] = byte_f(w.l, 1);
-    const uint32_t mid = a4 ? w.m0 : (w.m0 | (w.m1 << 16));
-    v[2] = byte_f(mid, 0);
-    v[3] = byte_f(mid, 1);
-    v[4] = byte_f(mid, 2);
-    v[5] = byte_f(mid, 3);
-    v[6] = byte_f(w.r, 0);
-    v[7] = byte_f(w.r, 1);
+// The taps of coefficient columns n and n+1 side by side: v[k] = pixels
+// (x+k, x+2+k), k = 0..3.  The byte-to-float trick of byte_f, two at a time.
+__device__ __forceinline__ void unpack_raw6(const Raw6 &w, bool a4, f32x2 *v) {
+    const uint32_t lo = a4 ? w.m0 : (w.m0 | (w.m1 << 16));
+    auto bits = [](uint32_t word, int k) { return __int_as_float(__byte_perm(word, 0x4B000000u, 0x7440u | (uint32_t)k)); };
+    const f32x2 off = pk2(-8388608.0f, -8388608.0f);
+    v[0] = add2(pk2(bits(lo, 0), bits(lo, 2)), off);
+    v[1] = add2(pk2(bits(lo, 1), bits(lo, 3)), off);
+    v[2] = add2(pk2(bits(lo, 2), bits(w.r, 0)), off);
+    v[3] = add2(pk2(bits(lo, 3), bits(w.r, 1)), off);
+}
+__device__ __forceinline__ void load_taps(const uint8_t *row, const LaneCols &c, bool a4, f32x2 *v) {
+    unpack_raw6(load_raw6(row, c, a4), a4, v);
+}
+__device__ __forceinline__ void load_taps(const float *row, const LaneCols &c, bool a4, f32x2 *v) {
+    float p[4], q[2];
+    load_row4(row, c, a4, p);
+    ld2(row + c.c4, q[0], q[1]);
+    v[0] = pk2(p[0], p[2]);
+    v[1] = pk2(p[1], p[3]);
+    v[2] = pk2(p[2], q[0]);
+    v[3] = pk2(p[3], q[1]);
 }
 
 // ------------------------------------------------------------------ output sinks
@@ -140,6 +141,11 @@ struct FwdDirect {
         float *p = Z + ((q < 2 ? m : H2 + m) + r) * W + ((q & 1) ? W2 : 0) + c.nB;
         store_pair(p, pair, c.two, a, b);
     }
+    __device__ __forceinline__ void quad(int64_t m, int r, int q, f32x2 v) const {
+        float a, b;
+        up2(v, a, b);
+        quad(m, r, q, a, b);
+    }
     __device__ __forceinline__ void step_end(int64_t, bool) const {}
 };
 
@@ -159,6 +165,10 @@ struct FwdStaged {
     __device__ __forceinline__ void quad(int64_t, int r, int q, float a, float b) const {
         if (!c.active) return;
         *reinterpret_cast<float2 *>(slot() + (r * 4 + q) * kSeg + (c.nB - n0)) = make_float2(a, b);
+    }
+    __device__ __forceinline__ void quad(int64_t, int r, int q, f32x2 v) const {
+        if (!c.active) return;
+        *reinterpret_cast<f32x2 *>(slot() + (r * 4 + q) * kSeg + (c.nB - n0)) = v;
     }
     __device__ __forceinline__ void step_end(int64_t m, bool second) const {
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -226,70 +236,78 @@ __device__ __forceinline__ void dwt2_item(const DwtArgs &s, int64_t x0, int64_t 
         }
         return;
     }
-    // D4: rows 2m .. 2m+3 (periodic) feed coefficient row m.
-    float a0[2], d0[2], a1[2], d1[2];
+    // D4: rows 2m .. 2m+3 (periodic) feed coefficient row m.  All sums in
+    // paired FP32 over the lane's two coefficient columns (n, n+1): the pass is
+    // bound by its instructions (ncu, staged: 71 % of issue slots).
+    const f32x2 h0 = pk2(kH0, kH0), h1 = pk2(kH1, kH1), h2 = pk2(kH2, kH2), h3 = pk2(kH3, kH3);
+    const f32x2 g0 = pk2(kG0, kG0), g1 = pk2(kG1, kG1), g2 = pk2(kG2, kG2), g3 = pk2(kG3, kG3);
+    f32x2 a0, d0, a1, d1;
+    auto low = [&](f32x2 x0v, f32x2 x1, f32x2 x2, f32x2 x3) { return fma2(h3, x3, fma2(h2, x2, fma2(h1, x1, mul2(h0, x0v)))); };
+    auto high = [&](f32x2 x0v, f32x2 x1, f32x2 x2, f32x2 x3) { return fma2(g3, x3, fma2(g2, x2, fma2(g1, x1, mul2(g0, x0v)))); };
+    auto row_ad = [&](const f32x2 *v, f32x2 &ra, f32x2 &rd) {
+        ra = low(v[0], v[1], v[2], v[3]);
+        rd = high(v[0], v[1], v[2], v[3]);
+    };
     {
-        float v[8];
-        load_row8(img + (2 * m_s) * W, c, a4, v);
-        d4_row_ad(v, a0, d0);
-        load_row8(img + (2 * m_s + 1) * W, c, a4, v);
-        d4_row_ad(v, a1, d1);
+        f32x2 v[4];
+        load_taps(img + (2 * m_s) * W, c, a4, v);
+        row_ad(v, a0, d0);
+        load_taps(img + (2 * m_s + 1) * W, c, a4, v);
+        row_ad(v, a1, d1);
     }
     // uint8 images: the raw words of the next step's two rows are loaded one
     // step ahead (a few registers), so a warp's loads overlap its arithmetic.
     constexpr bool kPrefetch = sizeof(T) == 1;
-    Raw8 na, nb;
+    const T *next = img + wrap(2 * m_s + 2, H) * W;  // the rows the current step adds
+    Raw6 na, nb;
     if constexpr (kPrefetch) {
-        na = load_raw8(img + wrap(2 * m_s + 2, H) * W, c, a4);
-        nb = load_raw8(img + wrap(2 * m_s + 3, H) * W, c, a4);
+        na = load_raw6(next, c, a4);
+        nb = load_raw6(next + W, c, a4);
     }
     for (int64_t m = m_s; m < m_e; ++m) {
-        float va[8], vb[8];
+        f32x2 va[4], vb[4];
+        const T *after = m + 2 == (H >> 1) ? img : next + 2 * W;  // past the last row comes row 0
         if constexpr (kPrefetch) {
-            const Raw8 ra = na, rb = nb;
+            const Raw6 ra = na, rb = nb;
             if (m + 1 < m_e) {
-                na = load_raw8(img + wrap(2 * m + 4, H) * W, c, a4);
-                nb = load_raw8(img + wrap(2 * m + 5, H) * W, c, a4);
+                na = load_raw6(after, c, a4);
+                nb = load_raw6(after + W, c, a4);
             }
-            unpack_raw8(ra, a4, va);
-            unpack_raw8(rb, a4, vb);
+            unpack_raw6(ra, a4, va);
+            unpack_raw6(rb, a4, vb);
         } else {
-            load_row8(img + wrap(2 * m + 2, H) * W, c, a4, va);
-            load_row8(img + wrap(2 * m + 3, H) * W, c, a4, vb);
+            load_taps(next, c, a4, va);
+            load_taps(next + W, c, a4, vb);
         }
-        float a2[2], d2[2], a3[2], d3[2];
-        d4_row_ad(va, a2, d2);
-        d4_row_ad(vb, a3, d3);
+        next = after;
+        f32x2 a2, d2, a3, d3;
+        row_ad(va, a2, d2);
+        row_ad(vb, a3, d3);
         if (c.active) {
-            float ll[2], lh[2], hl[2], hh[2];
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                ll[j] = fmaf(kH3, a3[j], fmaf(kH2, a2[j], fmaf(kH1, a1[j], kH0 * a0[j])));
-                lh[j] = fmaf(kG3, a3[j], fmaf(kG2, a2[j], fmaf(kG1, a1[j], kG0 * a0[j])));
-                hl[j] = fmaf(kH3, d3[j], fmaf(kH2, d2[j], fmaf(kH1, d1[j], kH0 * d0[j])));
-                hh[j] = fmaf(kG3, d3[j], fmaf(kG2, d2[j], fmaf(kG1, d1[j], kG0 * d0[j])));
-            }
-            sink.quad(m, 0, 0, ll[0], ll[1]);
-            sink.quad(m, 0, 1, hl[0], hl[1]);
-            sink.quad(m, 0, 2, lh[0], lh[1]);
-            sink.quad(m, 0, 3, hh[0], hh[1]);
+            sink.quad(m, 0, 0, low(a0, a1, a2, a3));
+            sink.quad(m, 0, 1, low(d0, d1, d2, d3));
+            sink.quad(m, 0, 2, high(a0, a1, a2, a3));
+            sink.quad(m, 0, 3, high(d0, d1, d2, d3));
         }
         sink.step_end(m, false);
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            a0[j] = a2[j]; d0[j] = d2[j];
-            a1[j] = a3[j]; d1[j] = d3[j];
-        }
+        a0 = a2; d0 = d2;
+        a1 = a3; d1 = d3;
     }
 }
 
 // Inverse.  Per coefficient row i the lane forms, at its 4 image columns,
 //   RA(i, .) = row synthesis of (LL, top-right) and RB(i, .) = of (bottom-left, HH),
 // then column synthesis mixes rows i = m and m-1 (D4) or row m alone (Haar).
-__device__ __forceinline__ void load_coef3(const float *row, const LaneCols &c, float *v) {
+__device__ __forceinline__ void load_coef3(const float *row, const LaneCols &c, bool pair, float *v) {
     v[0] = __ldg(row + c.nA);
-    v[1] = __ldg(row + c.nB);
-    v[2] = __ldg(row + c.nC);
+    if (pair) {
+        const float2 w = __ldg(reinterpret_cast<const float2 *>(row + c.nB));
+        v[1] = w.x;
+        v[2] = w.y;
+    } else {
+        v[1] = __ldg(row + c.nB);
+        v[2] = __ldg(row + c.nC);
+    }
 }
 
 // D4 row synthesis at image columns x..x+3 of a low-pass half L (h taps) and
@@ -342,25 +360,26 @@ __device__ __forceinline__ void idwt2_item(const DwtArgs &s, int64_t x0, int64_t
         }
         return;
     }
+    const bool pair = s.pairs != 0;
     float rap[4], rbp[4];  // RA, RB of coefficient row m-1
     {
         const int64_t mp = wrap(m_s - 1, H2);
         float L[3], G[3];
-        load_coef3(Z + mp * W, c, L);
-        load_coef3(Z + mp * W + W2, c, G);
+        load_coef3(Z + mp * W, c, pair, L);
+        load_coef3(Z + mp * W + W2, c, pair, G);
         d4_row_syn(L, G, rap);
-        load_coef3(Z + (H2 + mp) * W, c, L);
-        load_coef3(Z + (H2 + mp) * W + W2, c, G);
+        load_coef3(Z + (H2 + mp) * W, c, pair, L);
+        load_coef3(Z + (H2 + mp) * W + W2, c, pair, G);
         d4_row_syn(L, G, rbp);
     }
     // The next row's 12 coefficients are loaded one step ahead (the kernel
     // runs two CTAs per SM at its register count either way), so a warp's
     // loads overlap its arithmetic.
     float nL0[3], nG0[3], nL1[3], nG1[3];
-    load_coef3(Z + m_s * W, c, nL0);
-    load_coef3(Z + m_s * W + W2, c, nG0);
-    load_coef3(Z + (H2 + m_s) * W, c, nL1);
-    load_coef3(Z + (H2 + m_s) * W + W2, c, nG1);
+    load_coef3(Z + m_s * W, c, pair, nL0);
+    load_coef3(Z + m_s * W + W2, c, pair, nG0);
+    load_coef3(Z + (H2 + m_s) * W, c, pair, nL1);
+    load_coef3(Z + (H2 + m_s) * W + W2, c, pair, nG1);
     for (int64_t m = m_s; m < m_e; ++m) {
         float L0[3], G0[3], L1[3], G1[3];
 #pragma unroll
@@ -368,10 +387,10 @@ __device__ __forceinline__ void idwt2_item(const DwtArgs &s, int64_t x0, int64_t
             L0[k] = nL0[k]; G0[k] = nG0[k]; L1[k] = nL1[k]; G1[k] = nG1[k];
         }
         if (m + 1 < m_e) {
-            load_coef3(Z + (m + 1) * W, c, nL0);
-            load_coef3(Z + (m + 1) * W + W2, c, nG0);
-            load_coef3(Z + (H2 + m + 1) * W, c, nL1);
-            load_coef3(Z + (H2 + m + 1) * W + W2, c, nG1);
+            load_coef3(Z + (m + 1) * W, c, pair, nL0);
+            load_coef3(Z + (m + 1) * W + W2, c, pair, nG0);
+            load_coef3(Z + (H2 + m + 1) * W, c, pair, nL1);
+            load_coef3(Z + (H2 + m + 1) * W + W2, c, pair, nG1);
         }
         float ra[4], rb[4];
         d4_row_syn(L0, G0, ra);
