@@ -23,11 +23,12 @@
 // for the copies' reads, then release the slot) ran 5180-5330 GB/s on every
 // width.
 //
-// Used for single scenes (fuse_staged_applies) with rows on the 16-byte grid
-// (W % 4 == 0 with 16-byte-aligned float planes: every bulk copy starts on a
-// 16-byte boundary and moves a multiple of 16 bytes) and at most
+// Used for single scenes (fuse_staged_applies) in chunks of at most
 // kStagedMaxBands bands (two slots of 6 bands x 2 rows x 4 KB = 96 KB, two
-// CTAs per SM); the band-chunk knob splits them further.
+// CTAs per SM; the band-chunk knob splits them further).  A bulk copy starts
+// on a 16-byte boundary and moves a multiple of 16 bytes: rows on the 16-byte
+// grid go out whole; on shifted rows (W % 4 == 2) the slot's odd rows lie 2
+// floats in, and the pairs at a row segment's ends go out as plain stores.
 #include "fuse_tile.cuh"
 #include "launch.h"
 
@@ -41,13 +42,23 @@ constexpr int kStCols = kStWarps * kWarpCols;  // 1024 PAN columns per CTA strip
 
 __device__ __forceinline__ unsigned st_smem(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
+__device__ __forceinline__ void bulk_out(float *dst, const float *src, unsigned bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(dst), "r"(st_smem(src)), "r"(bytes)
+                 : "memory");
+}
 // The issuing threads' bulk copies have read their shared-memory source.
 __device__ __forceinline__ void bulk_wait_read() {
     asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
 }
 
-template <int NB>
+// Floats between the slot's rows: with SHIFT a row's pixels start 0 (even rows)
+// or 2 (odd rows) floats in, like the image row past its 16-byte boundary.
+template <bool SHIFT>
+constexpr int kStRow = kStCols + (SHIFT ? 8 : 0);
+
+template <int NB, bool SHIFT>
 struct StagedEmit {
+    static constexpr int kRow = kStRow<SHIFT>, kLay = SHIFT ? kShift : kVec;
     // Up to 4 bands: the next row's inputs loaded ahead (8192^2 x 3 208 -> 184
     // us).  More: scalar synthesis, and the uint8 pixels stored after the
     // float rows' copies are issued, behind the row barrier (16384^2 x 6 float
@@ -56,16 +67,17 @@ struct StagedEmit {
     static constexpr int kMode = NB > 4 ? kScalarCol | kScalarRow : kAheadPan | kAheadMs;
     const SceneArgs &s;
     const LaneCols &c;
-    float *buf;    // two slots of [NB][2][kStCols] floats
+    float *buf;    // two slots of [NB][2][kRow] floats
     int64_t X0;    // first column of the CTA strip
-    int ncols;     // columns of the strip inside the image (a multiple of 4)
+    int ncols;     // columns of the strip inside the image (even; a multiple of 4 but for SHIFT)
+    int lane;
     int b0;        // first band of the launch's chunk
     int *rowc;     // the CTA's row count: row k fills slot k & 1
     bool hu;       // uint8 output wanted
     uint8_t *u;    // its band b0, the current MS row's first image row, column x
     uint32_t w8[kLate ? NB : 1][2];  // kLate: the row's uint8 words
 
-    __device__ __forceinline__ float *slot() const { return buf + (*rowc & 1) * (NB * 2 * kStCols); }
+    __device__ __forceinline__ float *slot() const { return buf + (*rowc & 1) * (NB * 2 * kRow); }
 
     template <typename M>
     __device__ __forceinline__ void band(int b, const float *v0, const float *v1, M, M) {
@@ -77,16 +89,22 @@ struct StagedEmit {
         } else {
             u += b ? s.out_plane : 0;
         }
-        if (!c.active) return;
-        float *row = slot() + b * 2 * kStCols + (c.x - (int)X0);
-        *reinterpret_cast<float4 *>(row) = make_float4(v0[0], v0[1], v0[2], v0[3]);
-        *reinterpret_cast<float4 *>(row + kStCols) = make_float4(v1[0], v1[1], v1[2], v1[3]);
+        if (c.active) {
+            float *row = slot() + b * 2 * kRow + (c.x - (int)X0);
+            *reinterpret_cast<float4 *>(row) = make_float4(v0[0], v0[1], v0[2], v0[3]);
+            if (SHIFT) {
+                *reinterpret_cast<float2 *>(row + kRow + 2) = make_float2(v1[0], v1[1]);
+                *reinterpret_cast<float2 *>(row + kRow + 4) = make_float2(v1[2], v1[3]);
+            } else {
+                *reinterpret_cast<float4 *>(row + kRow) = make_float4(v1[0], v1[1], v1[2], v1[3]);
+            }
+        }
         if (!kLate && hu) store_rows(u, pack4u8(v0), pack4u8(v1));
     }
 
     __device__ __forceinline__ void store_rows(uint8_t *q, uint32_t w0, uint32_t w1) const {
-        store_u8<kVec>(q, c, 0, false, w0);
-        store_u8<kVec>(q + s.W, c, 0, true, w1);
+        store_u8<kLay>(q, c, lane, false, w0);
+        store_u8<kLay>(q + s.W, c, lane, true, w1);
     }
 
     template <int>
@@ -100,9 +118,23 @@ struct StagedEmit {
             const int b = t >> 1, r = t & 1;
             const int64_t y = 2 * (int64_t)(m - s.m_lo) + r;
             float *dst = s.out_f32 + (int64_t)(b0 + b) * s.out_plane + y * s.W + X0;
-            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(dst),
-                         "r"(st_smem(slot() + (b * 2 + r) * kStCols)), "r"((unsigned)ncols * 4u)
-                         : "memory");
+            const float *src = slot() + (b * 2 + r) * kRow;
+            if (SHIFT) {
+                // The pixel pairs before the first and after the last 16-byte
+                // boundary by plain stores, what lies between as one copy.
+                int n = ncols;
+                if (r) {
+                    *reinterpret_cast<float2 *>(dst) = *reinterpret_cast<const float2 *>(src + 2);
+                    dst += 2;
+                    src += 4;
+                    n -= 2;
+                }
+                if (n & 2)
+                    *reinterpret_cast<float2 *>(dst + (n & ~3)) = *reinterpret_cast<const float2 *>(src + (n & ~3));
+                if (n >= 4) bulk_out(dst, src, (unsigned)(n & ~3) * 4u);
+            } else {
+                bulk_out(dst, src, (unsigned)ncols * 4u);
+            }
             asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
         }
         if (kLate) {
@@ -124,7 +156,7 @@ struct StagedEmit {
 
 // One CTA item: columns [X0, X0 + 1024), MS rows [m_s, m_e), bands
 // [b0, b0 + NB).  Every thread of the CTA calls it, with the same row count.
-template <typename T, int WAV, int NB>
+template <typename T, int WAV, int NB, bool SHIFT>
 __device__ __forceinline__ void staged_item(const SceneArgs &s, float *buf, int64_t X0, int m_s, int m_e, int b0,
                                             int *rowc) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -132,8 +164,8 @@ __device__ __forceinline__ void staged_item(const SceneArgs &s, float *buf, int6
     const LaneCols c = lane_cols(x0, lane, s.W);  // warps past W: idle lanes
     const int ncols = (int)min((int64_t)kStCols, s.W - X0);
     uint8_t *u = s.out_u8 + (int64_t)b0 * s.out_plane + (int64_t)(2 * (m_s - s.m_lo)) * s.W + c.x;
-    StagedEmit<NB> out{s, c, buf, X0, ncols, b0, rowc, s.out_u8 != nullptr, u};
-    walk_rows<T, WAV, NB, kVec>(s, c, x0, m_s, m_e, b0, out);
+    StagedEmit<NB, SHIFT> out{s, c, buf, X0, ncols, lane, b0, rowc, s.out_u8 != nullptr, u};
+    walk_rows<T, WAV, NB, SHIFT ? kShift : kVec>(s, c, x0, m_s, m_e, b0, out);
 }
 
 __device__ __forceinline__ void bulk_drain() {
@@ -143,7 +175,7 @@ __device__ __forceinline__ void bulk_drain() {
 }  // namespace
 
 // Single scene, bands [b0, b0 + NB); CTA items it = blockIdx.x, + gridDim.x, ...
-template <typename T, int WAV, int NB>
+template <typename T, int WAV, int NB, bool SHIFT>
 __global__ void __launch_bounds__(kStThreads, 2)
 fuse_staged_kernel(const __grid_constant__ SceneArgs s, int b0, int64_t strips_cta, int64_t items, int R) {
     extern __shared__ __align__(128) float st_buf[];
@@ -151,44 +183,64 @@ fuse_staged_kernel(const __grid_constant__ SceneArgs s, int b0, int64_t strips_c
     for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
         const int64_t sx = it % strips_cta, sy = it / strips_cta;
         const int m_s = s.m_lo + (int)(sy * R);
-        staged_item<T, WAV, NB>(s, st_buf, sx * kStCols, m_s, min(m_s + R, s.m_hi), b0, &rowc);
+        staged_item<T, WAV, NB, SHIFT>(s, st_buf, sx * kStCols, m_s, min(m_s + R, s.m_hi), b0, &rowc);
     }
     bulk_drain();
 }
 
 namespace {
 
+template <typename T, int WAV, int NB>
+void *st_fn_nb(bool shift) {
+    return shift ? reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, NB, true>)
+                 : reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, NB, false>);
+}
+
 template <typename T, int WAV>
-void *st_fn(int nb) {
+void *st_fn(int nb, bool shift) {
     switch (nb) {
-        case 1: return reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, 1>);
-        case 2: return reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, 2>);
-        case 3: return reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, 3>);
-        case 4: return reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, 4>);
-        case 5: return reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, 5>);
-        case 6: return reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, 6>);
+        case 1: return st_fn_nb<T, WAV, 1>(shift);
+        case 2: return st_fn_nb<T, WAV, 2>(shift);
+        case 3: return st_fn_nb<T, WAV, 3>(shift);
+        case 4: return st_fn_nb<T, WAV, 4>(shift);
+        case 5: return st_fn_nb<T, WAV, 5>(shift);
+        case 6: return st_fn_nb<T, WAV, 6>(shift);
         default: return nullptr;
     }
 }
 
-constexpr int staged_smem(int nb) { return 2 * nb * 2 * kStCols * (int)sizeof(float); }
+constexpr int staged_smem(int nb, bool shift) {
+    return 2 * nb * 2 * (shift ? kStRow<true> : kStRow<false>) * (int)sizeof(float);
+}
 
 }  // namespace
 
 // The staged kernel pays where a CTA's 8 warps, which meet at a barrier every
-// MS row, rarely wait for one another: whole 1024-column strips (idle warps
-// in a ragged last strip are lost time), and at most kStagedMaxBands bands
-// (8 bands would run as two 4-band launches reading PAN twice, slower than
-// the warp kernel's one).  Measured against the warp kernel (float32 out,
-// bench.py --case fuse and single scenes of the 96-scene workload): 16384^2 x
-// 6 6168 -> 6538 GB/s, 16384 x 4092 x 6 5364 -> 6137, 4958 x 7932 x 6 5728 ->
-// 5728, 6408 x 2256 x 8 4875 -> 3804 (8 bands, a 3/4-empty last strip).  The
-// same CTA items in the batched launch ran slower than its warp items on
-// every scene class tried (46 scenes on the grid: 5356 -> 4651 GB/s; with the
-// next item fetched during the current one and 64-row items: 4644), so the
-// batched launch keeps warp items.
+// MS row, rarely wait for one another: nearly whole 1024-column strips (idle
+// warps in a ragged last strip are lost time).  Up to 6 bands on aligned rows:
+// at every size (16384 x 4092 x 6 5364 -> 6137 GB/s against the warp kernel).
+// Shifted rows, and uint8 scenes of more bands (balanced chunks of at most 6,
+// PAN read once per chunk): where the output is many times the L2
+// (kStagedLarge bytes); smaller ones run faster item by item.  us, warp ->
+// staged: 16384 x 16382 x 6 1789 -> 1542, 8190^2 x 8 560 -> 500, 8190^2 x 3 230
+// -> 197, 8192 x 8140 x 8 554 -> 504, 16384^2 x 8 1952 -> 1910, 8192^2 x 12 733
+// -> 675; below the line 3736 x 4070 x 3 47 -> 51, 3000 x 2998 x 5 48 -> 55,
+// 4096^2 x 8 float 102 -> 107.  Float scenes of more than 6 aligned bands read
+// four times the PAN bytes per chunk and stay on the warp kernel.  The same CTA
+// items in the batched launch ran slower than its warp items on every scene
+// class tried (46 scenes on the grid: 5356 -> 4651 GB/s; with the next item
+// fetched during the current one and 64-row items: 4644), so the batched
+// launch keeps warp items.
+constexpr int64_t kStagedLarge = 700000000;
+
 bool fuse_staged_applies(const SceneArgs &s) {
-    if (s.a4 == 0 || s.out_f32 == nullptr || s.bands > kStagedMaxBands) return false;
+    if ((s.a4 == 0 && s.alt == 0) || s.out_f32 == nullptr) return false;
+    const bool more = s.bands > kStagedMaxBands;
+    if (s.a4 == 0 || more) {
+        if (s.a4 != 0 && s.in_f32) return false;
+        const int64_t px = 2 * (int64_t)(s.m_hi - s.m_lo) * s.W * s.bands;
+        if (px * (s.out_u8 ? 5 : 4) < kStagedLarge) return false;
+    }
     const int64_t strips = (s.W + kStCols - 1) / kStCols;
     return (strips * kStCols - s.W) * 8 <= strips * kStCols;
 }
@@ -206,10 +258,11 @@ cudaError_t launch_fuse_staged(const SceneArgs &s, int R, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     for (int b0 = 0; b0 < s.bands; b0 += chunk) {
         const int nb = s.bands - b0 < chunk ? s.bands - b0 : chunk;
-        void *fn = s.in_f32 ? (s.wavelet ? st_fn<float, 1>(nb) : st_fn<float, 0>(nb))
-                            : (s.wavelet ? st_fn<uint8_t, 1>(nb) : st_fn<uint8_t, 0>(nb));
+        const bool shift = s.a4 == 0;
+        void *fn = s.in_f32 ? (s.wavelet ? st_fn<float, 1>(nb, shift) : st_fn<float, 0>(nb, shift))
+                            : (s.wavelet ? st_fn<uint8_t, 1>(nb, shift) : st_fn<uint8_t, 0>(nb, shift));
         if (fn == nullptr) return cudaErrorInvalidValue;
-        const int smem = staged_smem(nb);
+        const int smem = staged_smem(nb, shift);
         int occ = 0;
         e = resident_blocks_smem(fn, kStThreads, smem, &occ);
         if (e != cudaSuccess) return e;
