@@ -97,6 +97,9 @@ KNOWN_TRAFFIC: dict[str, float] = {
     # fixed-point partial rows:
     # read 706,983,424 + write 8,004,121,216 (mean of 2 launches)
     "aac3151ae716": 8711104640.0,
+    # an instance of the warp-strip emitter for a uint8 output alone (not this kernel's):
+    # read 709,886,976 + write 8,003,926,784 (mean of 2 launches)
+    "2c6e74a5403a": 8713813760.0,
 }
 KERNEL_SOURCES = ("fuse_tile.cuh", "fuse_metrics.cu", "metric_q.cuh", "tmem.cuh")
 

@@ -4,8 +4,6 @@
 
 namespace dwtfuse {
 
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
 constexpr int kAltMaxBands = 6;  // widest band chunk of the shifted-row instance
 // Shifted rows: neighbouring strips complete each other's sectors, and short
 // items bring them there close together (rows per item 4 against the balanced
@@ -14,57 +12,81 @@ constexpr int kAltMaxBands = 6;  // widest band chunk of the shifted-row instanc
 // float 520 -> 526).
 constexpr int kShiftRows = 4;
 
-// Walker mode (paired / scalar FP32 and loads ahead, us a call): up to 4 bands
-// PAN one row ahead (3736 x 4070 x 3 uint8 58 -> 53.5); more bands scalar
-// columns (8192^2 x 8 uint8 to float + uint8 502 -> 491, to uint8 alone 205 ->
-// 211), floats scalar rows too (8192^2 x 8 522 -> 493, 6 bands on shifted rows
-// 405 -> 398).
-template <typename T, int NB>
-constexpr int kFwdMode = NB <= 4 ? kAheadPan : (sizeof(T) == 4 ? kScalarCol | kScalarRow : kScalarCol);
+// Walker mode (paired / scalar FP32 and loads ahead, us a call) and CTA size of
+// an instance.  With a float output: up to 4 bands PAN one row ahead (3736 x
+// 4070 x 3 uint8 58 -> 53.5); more bands scalar columns (8192^2 x 8 uint8 to
+// float + uint8 502 -> 491), floats scalar rows too (8192^2 x 8 522 -> 493, 6
+// bands on shifted rows 405 -> 398).  A uint8 output alone leaves the walker
+// bound by instructions and load latency: paired FP32 and loads ahead as far as
+// the registers go, at 8192^2: 3 bands 109 -> 103, 5 bands 155 -> 134, 7 bands
+// 191 -> 175; 8 bands with 12 warps per SM whose registers hold the next row's
+// inputs (208 -> 194; 7480 x 8140 193 -> 174).
+template <typename T, int NB, bool U8ONLY>
+struct FwdShape {
+    static constexpr int kThreads = U8ONLY && NB == 8 ? 192 : 256;
+    static constexpr int kWarps = kThreads / 32;
+    static constexpr int kMode = U8ONLY    ? (NB <= 4 || NB == 8 ? kAheadPan | kAheadMs : NB <= 6 ? kAheadPan : 0)
+                                 : NB <= 4 ? kAheadPan
+                                           : (sizeof(T) == 4 ? kScalarCol | kScalarRow : kScalarCol);
+    // (8 bands: the walker without its float stores compiled to a slower
+    // schedule, 193 us against 174, so that instance keeps the run-time test)
+    static constexpr bool kNoFloat = U8ONLY && NB < 8;
+};
 
 // Single scene, bands [b0, b0 + NB).  Each warp takes work items
 // warp, warp + total_warps, ... (grid sized to the resident capacity).
-// Row layout: SHIFT kShift, else VEC kVec, else kPairs.
-template <typename T, int WAV, int NB, bool VEC, bool SHIFT>
-__global__ void __launch_bounds__(kThreads, 2)
+// Row layout: SHIFT kShift, else VEC kVec, else kPairs.  U8ONLY: a uint8
+// output and no float one.
+template <typename T, int WAV, int NB, bool U8ONLY, bool VEC, bool SHIFT>
+__global__ void __launch_bounds__(FwdShape<T, NB, U8ONLY>::kThreads, 2)
 fuse_fwd_kernel(const __grid_constant__ SceneArgs s, int b0, int64_t strips_x, int64_t items, int R) {
+    using F = FwdShape<T, NB, U8ONLY>;
     constexpr int LAY = SHIFT ? kShift : (VEC ? kVec : kPairs);
     const int lane = threadIdx.x & 31;
-    const int64_t nwarps = (int64_t)gridDim.x * kWarps;
-    for (int64_t it = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5); it < items; it += nwarps)
-        run_item<T, WAV, NB, LAY, kFwdMode<T, NB>>(s, it, strips_x, R, b0, lane);
+    const int64_t nwarps = (int64_t)gridDim.x * F::kWarps;
+    for (int64_t it = (int64_t)blockIdx.x * F::kWarps + (threadIdx.x >> 5); it < items; it += nwarps)
+        run_item<T, WAV, NB, LAY, F::kMode, F::kNoFloat>(s, it, strips_x, R, b0, lane);
 }
 
 // ------------------------------------------------------------------ host side
 
 namespace {
 
-template <typename T, int WAV, int NB>
-void *fwd_fn(int lay) {
-    if (lay == kVec) return reinterpret_cast<void *>(&fuse_fwd_kernel<T, WAV, NB, true, false>);
+struct FwdFn {
+    void *fn;
+    int threads;
+};
+
+template <typename T, int WAV, int NB, bool U8ONLY>
+FwdFn fwd_fn(int lay) {
+    constexpr int kT = FwdShape<T, NB, U8ONLY>::kThreads;
+    if (lay == kVec) return {reinterpret_cast<void *>(&fuse_fwd_kernel<T, WAV, NB, U8ONLY, true, false>), kT};
     if constexpr (NB <= kAltMaxBands)
-        if (lay == kShift) return reinterpret_cast<void *>(&fuse_fwd_kernel<T, WAV, NB, false, true>);
-    return lay == kPairs ? reinterpret_cast<void *>(&fuse_fwd_kernel<T, WAV, NB, false, false>) : nullptr;
+        if (lay == kShift) return {reinterpret_cast<void *>(&fuse_fwd_kernel<T, WAV, NB, U8ONLY, false, true>), kT};
+    if (lay == kPairs) return {reinterpret_cast<void *>(&fuse_fwd_kernel<T, WAV, NB, U8ONLY, false, false>), kT};
+    return {nullptr, 0};
 }
 
-template <typename T, int WAV>
-void *fwd_fn_nb(int nb, int lay) {
+template <typename T, int WAV, bool U8ONLY>
+FwdFn fwd_fn_nb(int nb, int lay) {
     switch (nb) {
-        case 1: return fwd_fn<T, WAV, 1>(lay);
-        case 2: return fwd_fn<T, WAV, 2>(lay);
-        case 3: return fwd_fn<T, WAV, 3>(lay);
-        case 4: return fwd_fn<T, WAV, 4>(lay);
-        case 5: return fwd_fn<T, WAV, 5>(lay);
-        case 6: return fwd_fn<T, WAV, 6>(lay);
-        case 7: return fwd_fn<T, WAV, 7>(lay);
-        case 8: return fwd_fn<T, WAV, 8>(lay);
-        default: return nullptr;
+        case 1: return fwd_fn<T, WAV, 1, U8ONLY>(lay);
+        case 2: return fwd_fn<T, WAV, 2, U8ONLY>(lay);
+        case 3: return fwd_fn<T, WAV, 3, U8ONLY>(lay);
+        case 4: return fwd_fn<T, WAV, 4, U8ONLY>(lay);
+        case 5: return fwd_fn<T, WAV, 5, U8ONLY>(lay);
+        case 6: return fwd_fn<T, WAV, 6, U8ONLY>(lay);
+        case 7: return fwd_fn<T, WAV, 7, U8ONLY>(lay);
+        case 8: return fwd_fn<T, WAV, 8, U8ONLY>(lay);
+        default: return {nullptr, 0};
     }
 }
 
-void *fwd_kernel_ptr(bool f32, int wav, int nb, int lay) {
-    if (f32) return wav ? fwd_fn_nb<float, 1>(nb, lay) : fwd_fn_nb<float, 0>(nb, lay);
-    return wav ? fwd_fn_nb<uint8_t, 1>(nb, lay) : fwd_fn_nb<uint8_t, 0>(nb, lay);
+FwdFn fwd_kernel(const SceneArgs &s, int nb, int lay) {
+    if (s.in_f32) return s.wavelet ? fwd_fn_nb<float, 1, false>(nb, lay) : fwd_fn_nb<float, 0, false>(nb, lay);
+    if (s.out_f32 == nullptr)
+        return s.wavelet ? fwd_fn_nb<uint8_t, 1, true>(nb, lay) : fwd_fn_nb<uint8_t, 0, true>(nb, lay);
+    return s.wavelet ? fwd_fn_nb<uint8_t, 1, false>(nb, lay) : fwd_fn_nb<uint8_t, 0, false>(nb, lay);
 }
 
 }  // namespace
@@ -84,10 +106,12 @@ cudaError_t launch_fuse(const SceneArgs &s, int R, int blocks_per_sm, cudaStream
     const int chunk = (alt || knob > 0) ? (s.bands + nchunks - 1) / nchunks : kChunkBands;
     for (int b0 = 0; b0 < s.bands; b0 += chunk) {
         const int nb = s.bands - b0 < chunk ? s.bands - b0 : chunk;
-        void *fn = fwd_kernel_ptr(s.in_f32 != 0, s.wavelet, nb, row_layout(s.a4, s.alt));
+        const FwdFn k = fwd_kernel(s, nb, row_layout(s.a4, s.alt));
+        void *fn = k.fn;
+        const int warps = k.threads / 32;
         if (fn == nullptr) return cudaErrorInvalidValue;
         int occ = 0;
-        cudaError_t e = resident_blocks(fn, kThreads, &occ);
+        cudaError_t e = resident_blocks(fn, k.threads, &occ);
         if (e != cudaSuccess) return e;
         if (blocks_per_sm > 0 && blocks_per_sm < occ) occ = blocks_per_sm;
         int sms = 0;
@@ -98,17 +122,17 @@ cudaError_t launch_fuse(const SceneArgs &s, int R, int blocks_per_sm, cudaStream
         const int64_t rows2 = 2 * (int64_t)(s.m_hi - s.m_lo);
         int Rl = R;
         if (Rl <= 0) {
-            Rl = balanced_rows((s.W + kWarpCols - 1) / kWarpCols, rows2 / 2, cap * kWarps);
+            Rl = balanced_rows((s.W + kWarpCols - 1) / kWarpCols, rows2 / 2, cap * warps);
             if (alt && Rl > kShiftRows) Rl = kShiftRows;
         }
         const ItemGrid g = item_grid(rows2, s.W, Rl);
-        const int64_t need = (g.items + kWarps - 1) / kWarps;
+        const int64_t need = (g.items + warps - 1) / warps;
         const unsigned grid = (unsigned)(need < cap ? need : cap);
         if (grid == 0) continue;
         SceneArgs sa = s;
         int64_t strips_x = g.strips_x, items = g.items;
         void *args[] = {&sa, (void *)&b0, &strips_x, &items, &Rl};
-        e = cudaLaunchKernel(fn, dim3(grid), dim3(kThreads), args, 0, stream);
+        e = cudaLaunchKernel(fn, dim3(grid), dim3(k.threads), args, 0, stream);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

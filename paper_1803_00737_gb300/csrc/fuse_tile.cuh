@@ -780,7 +780,8 @@ struct OutRun {
 // Every lane writes its own 4 pixels to global memory.  kVec: 4-pixel
 // vectors; kShift: even rows as vectors (the lane at x = W-2 pairs), odd rows
 // through store4_shifted; kPairs: pixel pairs.
-template <int LAY, int MODE>
+// U8ONLY: the instance for a uint8 output alone.
+template <int LAY, int MODE, bool U8ONLY>
 struct DirectEmit {
     static constexpr bool kAllLanes = LAY == kShift;
     static constexpr int kMode = MODE;
@@ -794,12 +795,12 @@ struct DirectEmit {
 
     template <typename M>
     __device__ __forceinline__ void band(int, const float *v0, const float *v1, M, M) {
-        if (o.hf) {
+        if (!U8ONLY && o.hf) {
             store_f32<LAY>(o.f, c, lane, false, v0);
             store_f32<LAY>(o.f + W, c, lane, true, v1);
             o.f += plane;
         }
-        if (o.hu) {
+        if (U8ONLY || o.hu) {
             store_u8<LAY>(o.u, c, lane, false, pack4u8(v0));
             store_u8<LAY>(o.u + W, c, lane, true, pack4u8(v1));
             o.u += plane;
@@ -807,16 +808,18 @@ struct DirectEmit {
     }
     template <int NB>
     __device__ __forceinline__ void row_end(int, uint32_t, uint32_t) {
-        o.next_row(2 * (int64_t)W - NB * plane);
+        const int64_t step = 2 * (int64_t)W - NB * plane;
+        if (!U8ONLY) o.f += step;
+        o.u += step;
     }
 };
 
 // One warp strip: 128 PAN columns from x0, MS rows [m_s, m_e), bands
 // [b0, b0 + NB), written directly.
-template <typename T, int WAV, int NB, int LAY, int MODE>
+template <typename T, int WAV, int NB, int LAY, int MODE, bool U8ONLY = false>
 __device__ __forceinline__ void direct_item(const SceneArgs &s, int64_t x0, int m_s, int m_e, int b0, int lane) {
     const LaneCols c = lane_cols(x0, lane, s.W);
-    DirectEmit<LAY, MODE> out(s, c, b0, m_s, lane);
+    DirectEmit<LAY, MODE, U8ONLY> out(s, c, b0, m_s, lane);
     walk_rows<T, WAV, NB, LAY>(s, c, x0, m_s, m_e, b0, out);
 }
 
@@ -834,12 +837,12 @@ __host__ __device__ inline ItemGrid item_grid(int64_t H, int64_t W, int R) {
 }
 
 // Runs work item `item` of a scene on the walkers of one row layout.
-template <typename T, int WAV, int NB, int LAY, int MODE>
+template <typename T, int WAV, int NB, int LAY, int MODE, bool U8ONLY = false>
 __device__ __forceinline__ void run_item(const SceneArgs &s, int64_t item, int64_t strips_x, int R, int b0, int lane) {
     const int64_t sx = item % strips_x, sy = item / strips_x;
     const int m_s = s.m_lo + (int)(sy * R);
     const int m_e = min(m_s + R, s.m_hi);
-    direct_item<T, WAV, NB, LAY, MODE>(s, sx * kWarpCols, m_s, m_e, b0, lane);
+    direct_item<T, WAV, NB, LAY, MODE, U8ONLY>(s, sx * kWarpCols, m_s, m_e, b0, lane);
 }
 
 }  // namespace dwtfuse

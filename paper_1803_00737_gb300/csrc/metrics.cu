@@ -588,7 +588,7 @@ __device__ __forceinline__ void write_partial(long long *out, const float *sq, c
 // slots): items go round the CTAs (with 1.5 items a warp, CTAs of consecutive
 // items left half of the SMs idle in the second round: 188 -> 156 us), the row
 // copies post one byte count instead of one per plane, and skip the clipping
-// where no row of the item can leave its plane (832 -> 700 instructions a row).
+// where no row of the item can leave its plane (832 -> 760 instructions a row).
 // The float order of a warp's Q sums is that of its items, as before.
 //
 // GEN = false: rows of every plane start on 16-byte boundaries (W % 16 == 0,
