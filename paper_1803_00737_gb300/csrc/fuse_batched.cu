@@ -15,12 +15,16 @@ constexpr int kSceneBytes = (int)((sizeof(SceneArgs) + 15) / 16 * 16);
 // 256..4096 px: 719 us a call against 730 with 16 warps at 128), float 16
 // warps with the next row's inputs loaded ahead (forward + backward of
 // 8 x 4096^2 x 4: 1086 us a pass against 1129 with 20 warps, where that
-// spills, and 1101 with 16 and no loads ahead).
+// spills, and 1101 with 16 and no loads ahead).  More bands, 16 warps: floats
+// with scalar synthesis (4 x 4096^2 x 8 570 -> 480 us a call, 8 x 2048^2 x 8
+// 298 -> 248; paired, the walker spills), uint8 paired with PAN ahead (24
+// uneven scenes to uint8 469 -> 464).
 template <typename T, int MAXB>
 struct BatchShape {
     static constexpr bool kNarrow = MAXB <= kBatchNarrowBands, kFloat = sizeof(T) == 4;
     static constexpr int kThreads = kNarrow && !kFloat ? 320 : 256;
-    static constexpr int kMode = kNarrow && kFloat ? kAheadPan | kAheadMs : 0;
+    static constexpr int kMode = kNarrow ? (kFloat ? kAheadPan | kAheadMs : 0)
+                                         : (kFloat ? kScalarCol | kScalarRow : kAheadPan);
     static constexpr int kSmem = kThreads / 32 * kSceneBytes;
 };
 
