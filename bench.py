@@ -100,6 +100,9 @@ KNOWN_TRAFFIC: dict[str, float] = {
     # an instance of the warp-strip emitter for a uint8 output alone (not this kernel's):
     # read 709,886,976 + write 8,003,926,784 (mean of 2 launches)
     "2c6e74a5403a": 8713813760.0,
+    # adjacent strips of shifted rows of 5-7 bands in one CTA (the aligned 6-band body unchanged):
+    # read 706,875,008 + write 8,003,992,704 (mean of 2 launches)
+    "04090a8ee8f9": 8710867712.0,
 }
 KERNEL_SOURCES = ("fuse_tile.cuh", "fuse_metrics.cu", "metric_q.cuh", "tmem.cuh")
 

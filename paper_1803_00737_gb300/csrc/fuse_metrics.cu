@@ -69,6 +69,13 @@ struct FmLayout {
     // bands 12 warps at up to 168 (the 8-band walker spills at 128).
     static constexpr int kThreads = NB <= 7 ? 512 : 384;
     static constexpr int kWarps = kThreads / 32;
+    // Shifted rows of 5-7 bands, when every warp has an item: adjacent strips,
+    // which complete each other's sectors, in one CTA (8190^2 x 6 496 -> 462
+    // us, 11000 x 9998 x 6 857 -> 746, x 7 1022 -> 884, x 5 625 -> 613; not 3-4
+    // bands, 493 -> 512, nor 8, 945 -> 966).  Which SM a warp's items run on
+    // does not change its sums.
+    template <int LAY>
+    static constexpr bool kAdjacent = LAY == kShift && NB >= 5 && NB <= 7;
     // Per-warp shared memory (32-bit words, lane-minor so that lane accesses are conflict-free).
     static constexpr int kTile = K * 2 * SR * 32;     // uint8 words of 2 SR PAN rows: bands, PAN
     static constexpr int kRep = NB * SR * 32;         // MS reference words of SR MS rows
@@ -281,9 +288,12 @@ fuse_metrics_kernel(const __grid_constant__ SceneArgs s, double *partial, int st
         *tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * L::kWarpTmem);
 
     // Items go round the CTAs first (warp w of CTA b starts at item w G + b,
-    // G CTAs), so a scene with fewer items than warps still spreads over every SM.
+    // G CTAs), so a scene with fewer items than warps still spreads over every SM;
+    // kAdjacent: adjacent items in one CTA (the same items for the same virtual warp).
     const int64_t nwarps = (int64_t)gridDim.x * L::kWarps;
-    for (int64_t it = (int64_t)warp * gridDim.x + blockIdx.x; it < items; it += nwarps) {
+    const int64_t first = L::template kAdjacent<LAY> && items >= nwarps ? (int64_t)blockIdx.x * L::kWarps + warp
+                                                                        : (int64_t)warp * gridDim.x + blockIdx.x;
+    for (int64_t it = first; it < items; it += nwarps) {
         const int64_t sx = it % strips_x, sy = it / strips_x;
         const int64_t x0 = sx * kWarpCols;
         const int m_s = (int)(sy * R);
