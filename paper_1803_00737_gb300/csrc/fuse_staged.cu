@@ -51,6 +51,15 @@ __device__ __forceinline__ void bulk_wait_read() {
     asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
 }
 
+// The CTA's row barrier.  An emitter's row_end is instantiated in the inner-strip
+// and the edge-strip walker, and the warps of one CTA run both: every thread
+// (idle lanes too) arrives once per MS row, at one of several barrier
+// instructions.  PTX counts the arrivals per barrier number, whichever
+// instruction they come from, and without .aligned asks nothing of a warp's
+// convergence; __syncthreads() is defined only where the whole block takes the
+// same side of every condition around it.
+__device__ __forceinline__ void row_barrier() { asm volatile("barrier.sync 0;\n" ::: "memory"); }
+
 // Floats between the slot's rows: with SHIFT a row's pixels start 0 (even rows)
 // or 2 (odd rows) floats in, like the image row past its 16-byte boundary.
 template <bool SHIFT>
@@ -113,7 +122,7 @@ struct StagedEmit {
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         const int t = threadIdx.x;
         if (t < 2 * NB) bulk_wait_read();  // row m-1's copies: the slot row m+1 will fill
-        __syncthreads();
+        row_barrier();
         if (t < 2 * NB) {
             const int b = t >> 1, r = t & 1;
             const int64_t y = 2 * (int64_t)(m - s.m_lo) + r;
