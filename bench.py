@@ -88,21 +88,9 @@ KNOWN_TRAFFIC: dict[str, float] = {
     # the same kernel waiting for its TMEM stores before every scoring:
     # read 689,644,885 + write 7,989,676,288 (mean of 3 launches)
     "22e4d6d25dce": 8679321173.0,
-    # walkers with paired FP32 and running addresses:
-    # read 708,970,496 + write 8,006,513,664 (mean of 2 launches)
-    "686a90346174": 8715484160.0,
-    # row heights per launch, scalar synthesis where registers are short:
-    # read 709,261,440 + write 8,006,737,536 (mean of 2 launches)
-    "4ac0e872cfb0": 8715998976.0,
-    # fixed-point partial rows:
-    # read 706,983,424 + write 8,004,121,216 (mean of 2 launches)
-    "aac3151ae716": 8711104640.0,
-    # an instance of the warp-strip emitter for a uint8 output alone (not this kernel's):
-    # read 709,886,976 + write 8,003,926,784 (mean of 2 launches)
-    "2c6e74a5403a": 8713813760.0,
-    # adjacent strips of shifted rows of 5-7 bands in one CTA (the aligned 6-band body unchanged):
-    # read 706,875,008 + write 8,003,992,704 (mean of 2 launches)
-    "04090a8ee8f9": 8710867712.0,
+    # walkers with paired FP32 and running addresses, Q sums in two exact integers:
+    # read 707,550,037 + write 8,003,697,323 (mean of 3 launches)
+    "77b99d3ecf17": 8711247360.0,
 }
 KERNEL_SOURCES = ("fuse_tile.cuh", "fuse_metrics.cu", "metric_q.cuh", "tmem.cuh")
 

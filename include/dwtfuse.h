@@ -176,7 +176,9 @@ int dwtfuse_fuse_backward(const float *grad_out, int bands, int64_t H, int64_t W
  *   workspace dwtfuse_metrics_workspace_size() bytes of device memory, 8-byte
  *             aligned; its contents are scratch between calls
  * bands <= DWTFUSE_METRIC_MAX_BANDS (8).  QNR needs H/2, W/2 >= window.
- * Results are deterministic (fixed reduction order).
+ * Results are deterministic (fixed reduction order).  uint8 product and inputs:
+ * a warp's windows are added in FP32, those sums exactly (integers of units
+ * 2^-77), for any image the sides' limit of 2^20 allows.
  */
 #define DWTFUSE_QNR_WINDOW 32
 #define DWTFUSE_METRIC_MAX_BANDS 8

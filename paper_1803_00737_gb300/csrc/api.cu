@@ -458,7 +458,7 @@ int dwtfuse_fuse_and_score(const void *pan, const void *const *ms, int bands, in
                                    ws_bytes, &s, &m);
     if (st != DWTFUSE_OK) return st;
     if (!fuse_metrics_supported(s)) return DWTFUSE_ESHAPE;
-    return cuda_status(launch_fuse_metrics(s, m.workspace + kMetricPanPartialOffset, kMetricStride,
+    return cuda_status(launch_fuse_metrics(s, m.workspace + kMetricPanPartialOffset, metric_stride(bands),
                                            reinterpret_cast<int *>(m.workspace + kMetricPanCtasSlot),
                                            static_cast<cudaStream_t>(stream)));
 }
@@ -492,7 +492,7 @@ int dwtfuse_fuse_metrics(const void *pan, const void *const *ms, int bands, int6
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     cudaError_t e;
     if (fuse_metrics_supported(s)) {
-        e = launch_fuse_metrics(s, m.workspace + kMetricPanPartialOffset, kMetricStride,
+        e = launch_fuse_metrics(s, m.workspace + kMetricPanPartialOffset, metric_stride(bands),
                                 reinterpret_cast<int *>(m.workspace + kMetricPanCtasSlot), cs);
         m.pan_done = 1;
         m.ms_early = 1;  // the MS pass follows our own fused kernel directly

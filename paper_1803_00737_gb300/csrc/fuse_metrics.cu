@@ -313,23 +313,26 @@ fuse_metrics_kernel(const __grid_constant__ SceneArgs s, double *partial, int st
     // One partial row per CTA, in the layout of the PAN-resolution pass: Q sums
     // of the P pairs, then the NB squared-error sums.
     long long *outp = reinterpret_cast<long long *>(partial) + (int64_t)blockIdx.x * stride;
-    // One warp per entry at a time, as integers (fixed-point Q sums, exact
-    // squared errors: FP64 adds run at 2 lanes a clock).
+    // One warp per entry at a time, as exact integers (FP64 adds run at 2 lanes a
+    // clock).
     for (int k = warp; k < L::P + NB; k += L::kWarps) {
-        long long t = 0;
+        QSum t;
         if (k < L::P) {
             for (int i = lane; i < 4 * L::kWarps; i += 32) {
                 const float *qw = reinterpret_cast<const float *>(fm_smem + (i >> 2) * L::kWarpBytes) + L::kTile +
                                   L::kRep + L::kGsum;
-                t += __float2ll_rn(qw[(i & 3) * L::P + k] * (float)(1ll << kQFracBits));
+                t.add(qw[(i & 3) * L::P + k]);
             }
         } else {
             for (int w = 0; w < L::kWarps; ++w)
-                t += reinterpret_cast<const long long *>(fm_smem + w * L::kWarpBytes +
-                                                         L::kWords * 4)[(k - L::P) * 32 + lane];
+                t.hi += reinterpret_cast<const long long *>(fm_smem + w * L::kWarpBytes +
+                                                            L::kWords * 4)[(k - L::P) * 32 + lane];
         }
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0) outp[k] = t;
+        t.warp_sum();
+        if (lane == 0) {
+            outp[k] = t.hi;
+            if (k < L::P) outp[metric_lo_column(NB) + k] = t.lo;
+        }
     }
 }
 
@@ -392,7 +395,7 @@ cudaError_t launch_fuse_metrics(const SceneArgs &s, double *pan_partial, int str
     const ItemGrid g = item_grid(s.H, s.W, R);
     int64_t grid = g.items;  // every resident CTA, unless there are fewer items
     if (grid > cap) grid = cap;
-    if (grid > kMetricMaxCtas) grid = kMetricMaxCtas;
+    if (grid > metric_max_ctas(s.bands)) grid = metric_max_ctas(s.bands);
     if (grid < 1) grid = 1;
     SceneArgs sa = s;
     int64_t strips_x = g.strips_x, items = g.items;

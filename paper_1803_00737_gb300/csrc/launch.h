@@ -29,14 +29,17 @@ struct BatchTable {
 static_assert(sizeof(BatchTable) + 16 <= 32764, "batched scene table exceeds the parameter limit");
 
 // Quality metrics (metrics.cu).  Workspace layout, in doubles: 8 result slots
-// (ERGAS, QNR, D_lambda, D_s, ...), then kMetricMaxCtas partial rows of
-// kMetricStride for the PAN-resolution pass and as many for the MS pass.
-constexpr int kMetricMaxCtas = 1024;
-constexpr int kMetricStride = 64;    // >= pairs + bands for 8 bands (36 + 8)
-constexpr int kQFracBits = 40;       // fixed-point Q sums of the 8-bit passes' partial rows
+// (ERGAS, QNR, D_lambda, D_s, ...), then kMetricRoom for the partial rows of
+// the PAN-resolution pass and as many for the MS pass.  A row has 64 entries
+// (up to 7 bands: 2 * 28 pairs + 7 sums + 1 status), 128 for 8 bands.
+constexpr int64_t kMetricRoom = 65536;
+constexpr int kMetricCols = 64;      // >= pairs + bands + 1 for 8 bands (36 + 8 + 1)
+constexpr int kMetricIntCols = 81;   // entries of an int64 row of 8 bands: 2 * 36 + 8 + 1
+constexpr int metric_stride(int bands) { return bands <= 7 ? 64 : 128; }
+constexpr int metric_max_ctas(int bands) { return (int)(kMetricRoom / metric_stride(bands)); }
 constexpr int kMetricMaxBands = 8;
 constexpr int kMetricWindow = 32;
-constexpr size_t kMetricWorkspaceBytes = sizeof(double) * (8 + 2 * (size_t)kMetricMaxCtas * kMetricStride);
+constexpr size_t kMetricWorkspaceBytes = sizeof(double) * (8 + 2 * (size_t)kMetricRoom);
 
 struct MetricLaunch {
     const void *fused;

@@ -38,4 +38,42 @@ __device__ __forceinline__ float q_exact(long long sx, long long sxx, long long 
     return 4.0f * fc * fax * fay / den;
 }
 
+// Sum of windows' Q values (FP32), exact: the integers hi and lo, in units of
+// 2^-32 and 2^-77.  A window's Q is 0 or at least 2^-54 in size: the least is a
+// y of one quarter grey level (4 PAN~ = 1 in one pixel; cov = 1/4 in units of
+// n^2) against an x of mean m and the largest variance m (255 - m), which gives
+// 1 / (4 n^3 m^2 (255 - m)) > 2^-53.3.  So every Q, and every FP32 sum of them,
+// is a multiple of 2^-77.  Room: the largest images hold 2^30 windows (sides of
+// 2^20), |hi| <= 2^62; an addend's lo is below 2^45, and a pass adds at most
+// 1024 CTAs x 256 slots = 2^18 of them.  From the float's bits: conversions to
+// 64 bits and FP64 adds run at a few lanes a clock and SM (a CTA's 256 slots of
+// 21 pairs through three __float2ll_rn: 3 us at the end of the PAN pass).
+struct QSum {
+    long long hi = 0, lo = 0;
+    __device__ __forceinline__ void add(float q) {
+        const uint32_t w = __float_as_uint(q);
+        const int s = (int)((w >> 23) & 255u) - 73;  // q = +-m * 2^(s - 77)
+        if (s < 0) return;                           // 0
+        const unsigned long long m = (w & 0x7fffffu) | 0x800000u;
+        const long long h = (long long)(s >= 45 ? m << (s - 45) : m >> (45 - s));
+        const long long l = s >= 45 ? 0ll : (long long)((m << s) & ((1ull << 45) - 1));
+        hi += (w >> 31) ? -h : h;
+        lo += (w >> 31) ? -l : l;
+    }
+    __device__ __forceinline__ void warp_sum() {
+        for (int o = 16; o > 0; o >>= 1) {
+            hi += __shfl_xor_sync(0xffffffffu, hi, o);
+            lo += __shfl_xor_sync(0xffffffffu, lo, o);
+        }
+    }
+};
+__device__ __forceinline__ double q_value(long long hi, long long lo) {
+    return (double)hi * 0x1p-32 + (double)lo * 0x1p-77;
+}
+
+// Columns of a CTA's partial row, 8-bit passes (int64): the P pairs' QSum::hi,
+// nb sums (squared errors, MS values), the status of the bulk-copy waits, the
+// P pairs' QSum::lo.
+__host__ __device__ constexpr int metric_lo_column(int nb) { return nb * (nb + 1) / 2 + nb + 1; }
+
 }  // namespace dwtfuse

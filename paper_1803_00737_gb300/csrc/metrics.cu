@@ -22,10 +22,11 @@
 // exact integer (FP32 up to 2^24 in the PAN pass; int32 in the MS pass, where
 // PAN~ is carried as 4 * PAN~, an integer), the numerators n*Sxy - Sx*Sy and
 // n*Sxx - Sx^2 are formed exactly in int64, and only the final ratio is FP32
-// (relative error ~5e-7 per window).  Float data sum in FP32 and form the
-// numerators in FP64.  Per-window Q values are accumulated in FP64 in shared
-// memory; per-CTA partials go to the caller's workspace and a one-CTA kernel
-// reduces them in a fixed order (deterministic).
+// (relative error ~5e-7 per window); a warp adds its windows' Q in FP32 slots in
+// shared memory, and the slots are summed exactly (QSum, metric_q.cuh).  Float
+// data sum in FP32, form the numerators in FP64 and add Q in FP64.  Per-CTA
+// partials go to the caller's workspace and a one-CTA kernel reduces them in a
+// fixed order (deterministic).
 #include <type_traits>
 
 #include "fuse_tile.cuh"
@@ -559,24 +560,28 @@ struct FastPan {
     static constexpr int kSmem = kBarOffset + kFastWarps * kStages * 8;  // with the mbarriers (GEN)
 };
 
-// Partial rows of the 8-bit passes are int64: Q sums in units of 2^-kQFracBits,
-// squared errors and MS sums exact.  FP64 runs at 2 lanes a clock on an SM, and
-// adding a CTA's 256 Q values per pair and up to 456 rows of doubles in the
-// finalize was most of a small call: 512^2 x 3 57 -> 30 us with integers, the
-// finalize alone (ncu) 18 -> 12 us.
-__device__ __forceinline__ long long q_fixed(float q) { return __float2ll_rn(q * (float)(1ll << kQFracBits)); }
+// Partial rows of the 8-bit passes are int64, all sums exact (QSum of
+// metric_q.cuh; squared errors, MS sums).  FP64 runs at 2 lanes a clock on an
+// SM, and adding a CTA's 256 Q values per pair and up to 456 rows of doubles in
+// the finalize was most of a small call: 512^2 x 3 57 -> 31 us with integers,
+// the finalize alone (ncu) 18 -> 13 us (one int64 in units of 2^-40 per Q sum,
+// which wraps from 2^23 windows and loses Qs below it, ran 0.5-1 us faster, of 8
+// bands 3-5 us).
 
 // The CTA's partial row from the warps' Q slots (sq: [warps][windows][P]
 // floats) and sums (sum: [warps][NB] doubles, exact integers).  One warp per
-// pair at a time: its lanes add the slots (in a fixed order), then a butterfly.
+// pair at a time: its lanes add the slots, then a butterfly.
 template <int P, int NB, int WARPS>
 __device__ __forceinline__ void write_partial(long long *out, const float *sq, const double *sum) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int k = warp; k < P; k += WARPS) {
-        long long a = 0;
-        for (int s = lane; s < WARPS * kWinPerStrip; s += 32) a += q_fixed(sq[s * P + k]);
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (lane == 0) out[k] = a;
+        QSum a;
+        for (int s = lane; s < WARPS * kWinPerStrip; s += 32) a.add(sq[s * P + k]);
+        a.warp_sum();
+        if (lane == 0) {
+            out[k] = a.hi;
+            out[metric_lo_column(NB) + k] = a.lo;
+        }
     }
     if (threadIdx.x < NB) {
         long long a = 0;
@@ -1232,57 +1237,72 @@ metrics_ms_kernel(const __grid_constant__ MetricArgs a) {
 // exists at either resolution; all four NaN when a pass flagged in
 // `status_mask` (bit 0 PAN-resolution, bit 1 MS) reported a wait that gave up
 // in entry P + nb of a partial row), to `out` and, where given, `result`.
-// Thread (g, k) adds column k of rows g, g + 16, ...: 64 threads read a row's
-// 512 bytes together; then 16 sums per column (a fixed order, so the result is
-// the same on every run).  fixed_mask: passes whose rows are int64.
-constexpr int kFinalizeGroups = 16;
-constexpr int kFinalizeThreads = kFinalizeGroups * kMetricStride;
+// Thread (g, k) adds column k of rows g, g + G, ...: G groups of threads, as many
+// as a row has entries (64 for FP64 rows, whose sums keep their order), read
+// whole rows; then G sums per column (a fixed order, so the result is the same
+// on every run).  fixed_mask: passes whose rows are int64.
+constexpr int kFinalizeThreads = 1024;
+constexpr int kDoubleGroups = kFinalizeThreads / kMetricCols;
 template <typename S>
-__device__ __forceinline__ S column_sum(const double *part, int ctas, int g, int k) {
+__device__ __forceinline__ S column_sum(const double *part, int ctas, int stride, int groups, int g, int k) {
     const S *p = reinterpret_cast<const S *>(part) + k;
     S a = 0;
-#pragma unroll 8
-    for (int c = g; c < ctas; c += kFinalizeGroups) a += p[(int64_t)c * kMetricStride];
+    for (int c = g; c < ctas; c += 8 * groups) {  // eight rows' loads in flight, also in the last round
+        S v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int r = c + j * groups;
+            v[j] = r < ctas ? p[(int64_t)r * stride] : S(0);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) a += v[j];
+    }
     return a;
 }
 __global__ void __launch_bounds__(kFinalizeThreads)
 metrics_finalize_kernel(const double *pan_part, const double *ms_part, int ctas_pan, const int *ctas_pan_dev,
-                        int ctas_ms, int nb, int want_q, int64_t H, int64_t W, int64_t nwin_pan,
+                        int ctas_ms, int stride, int nb, int want_q, int64_t H, int64_t W, int64_t nwin_pan,
                         int64_t nwin_ms, int status_mask, int fixed_mask, double *out, double *result) {
     wait_primary();  // programmatic dependent of the MS-resolution pass
     if (ctas_pan_dev) ctas_pan = *ctas_pan_dev;
-    __shared__ double part[2][kFinalizeGroups][kMetricStride];  // (int64 bits of a fixed-point pass)
-    __shared__ double tot_pan[kMetricStride];
-    __shared__ double tot_ms[kMetricStride];
-    const int P = nb * (nb - 1) / 2 + nb;
+    __shared__ double part[2][kFinalizeThreads];  // [pass][group][column] (int64 bits of an int64 pass)
+    __shared__ long long col[2][kMetricIntCols];
+    __shared__ double tot_pan[kMetricCols];
+    __shared__ double tot_ms[kMetricCols];
+    const int P = nb * (nb - 1) / 2 + nb, LO = metric_lo_column(nb);
     const int lane = threadIdx.x & 31;
-    {
-        const int g = threadIdx.x / kMetricStride, k = threadIdx.x % kMetricStride;
+    const int groups = stride == kMetricCols ? kDoubleGroups : kDoubleGroups / 2;
 #pragma unroll
-        for (int ms = 0; ms < 2; ++ms) {
-            const bool used = k < P + nb || (k == P + nb && ((status_mask >> ms) & 1));
-            const int ctas = used ? (ms ? ctas_ms : ctas_pan) : 0;
-            const double *src = ms ? ms_part : pan_part;
-            if ((fixed_mask >> ms) & 1)
-                part[ms][g][k] = __longlong_as_double(column_sum<long long>(src, ctas, g, k));
-            else
-                part[ms][g][k] = column_sum<double>(src, ctas, g, k);
+    for (int ms = 0; ms < 2; ++ms) {
+        const bool fixed = (fixed_mask >> ms) & 1;
+        const int wide = fixed && stride != kMetricCols;  // 128 entries a row
+        const int g = (threadIdx.x / kMetricCols) >> wide, k = threadIdx.x & ((kMetricCols << wide) - 1);
+        const bool used = k == P + nb ? ((status_mask >> ms) & 1) != 0 : k < (fixed ? LO + P : P + nb);
+        const int ctas = used ? (ms ? ctas_ms : ctas_pan) : 0;
+        const double *src = ms ? ms_part : pan_part;
+        part[ms][threadIdx.x] =
+            fixed ? __longlong_as_double(column_sum<long long>(src, ctas, stride, groups, g, k))
+                  : column_sum<double>(src, ctas, stride, kDoubleGroups, g, k);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * stride) {
+        const int ms = threadIdx.x >= stride, k = threadIdx.x - ms * stride;
+        if ((fixed_mask >> ms) & 1) {
+            long long a = 0;
+#pragma unroll 8
+            for (int g = 0; g < groups; ++g) a += __double_as_longlong(part[ms][g * stride + k]);
+            if (k < kMetricIntCols) col[ms][k] = a;
+        } else if (k < kMetricCols) {
+            double t = 0.0;
+            for (int g = 0; g < kDoubleGroups; ++g) t += part[ms][g * kMetricCols + k];
+            (ms ? tot_ms : tot_pan)[k] = t;
         }
     }
     __syncthreads();
-    if (threadIdx.x < 2 * kMetricStride) {
-        const int ms = threadIdx.x / kMetricStride, k = threadIdx.x % kMetricStride;
-        double t;
-        if ((fixed_mask >> ms) & 1) {
-            long long a = 0;
-#pragma unroll
-            for (int g = 0; g < kFinalizeGroups; ++g) a += __double_as_longlong(part[ms][g][k]);
-            t = k < P ? (double)a * (1.0 / (double)(1ll << kQFracBits)) : (double)a;
-        } else {
-            t = 0.0;
-            for (int g = 0; g < kFinalizeGroups; ++g) t += part[ms][g][k];
-        }
-        (ms ? tot_ms : tot_pan)[k] = t;
+    if (threadIdx.x < 2 * kMetricCols) {
+        const int ms = threadIdx.x / kMetricCols, k = threadIdx.x % kMetricCols;
+        if (((fixed_mask >> ms) & 1) && k <= P + nb)
+            (ms ? tot_ms : tot_pan)[k] = k < P ? q_value(col[ms][k], col[ms][LO + k]) : (double)col[ms][k];
     }
     __syncthreads();
     if (threadIdx.x >= 32) return;
@@ -1381,14 +1401,13 @@ FastFn fast_fn(bool ms_pass, int nb, bool aligned) {
 }
 
 // Grid of a fast-path kernel: the resident CTAs (the row rings use most of
-// shared memory), at most kMetricMaxCtas, fewer with fewer items.  spread:
+// shared memory), at most metric_max_ctas, fewer with fewer items.  spread:
 // the kernel takes its items round the CTAs first and gets one CTA per item up
 // to that cap, so a scene with fewer items than warps still reaches every SM
 // (the MS-resolution pass: 8190^2 x 8 0.135 -> 0.119 ms, 16382^2 x 8 0.307 ->
 // 0.270 ms; the PAN-resolution pass, whose CTAs each end with a wide partial
 // row, ran slower that way and keeps items / warps CTAs).
-cudaError_t fast_grid(const FastFn &f, int64_t items, int *grid, bool spread = false) {
-    static_assert(kMetricMaxCtas >= 1, "");
+cudaError_t fast_grid(const FastFn &f, int64_t items, int bands, int *grid, bool spread = false) {
     int occ = 0, sms = 0;
     cudaError_t e = resident_blocks_smem(f.fn, f.warps * 32, f.smem, &occ);
     if (e != cudaSuccess) return e;
@@ -1397,7 +1416,7 @@ cudaError_t fast_grid(const FastFn &f, int64_t items, int *grid, bool spread = f
     int64_t g = spread ? items : (items + f.warps - 1) / f.warps;
     const int64_t cap = (int64_t)sms * occ;
     if (g > cap) g = cap;
-    if (g > kMetricMaxCtas) g = kMetricMaxCtas;
+    if (g > metric_max_ctas(bands)) g = metric_max_ctas(bands);
     if (g < 1) g = 1;
     *grid = (int)g;
     return cudaSuccess;
@@ -1417,7 +1436,7 @@ const void *ms_fn_nb(int nb) {
     }
 }
 
-cudaError_t grid_for(const void *fn, int64_t items, int *grid) {
+cudaError_t grid_for(const void *fn, int64_t items, int bands, int *grid) {
     int occ = 0, sms = 0;
     cudaError_t e = resident_blocks(fn, kMThreads, &occ);
     if (e != cudaSuccess) return e;
@@ -1426,7 +1445,7 @@ cudaError_t grid_for(const void *fn, int64_t items, int *grid) {
     int64_t g = (items + kMWarps - 1) / kMWarps;
     const int64_t cap = (int64_t)sms * occ;
     if (g > cap) g = cap;
-    if (g > kMetricMaxCtas) g = kMetricMaxCtas;
+    if (g > metric_max_ctas(bands)) g = metric_max_ctas(bands);
     if (g < 1) g = 1;
     *grid = (int)g;
     return cudaSuccess;
@@ -1445,12 +1464,12 @@ cudaError_t launch_metrics(const MetricLaunch &m, cudaStream_t stream) {
     a.want_q = m.want_q;
     a.a4_fused = m.a4_fused;
     a.a4_in = m.a4_in;
-    a.stride = kMetricStride;
+    a.stride = metric_stride(m.bands);
     a.wait_test = m.wait_test;
     const bool fast = !m.fused_f32 && !m.in_f32;
     double *out = m.workspace;
     double *pan_part = m.workspace + kMetricPanPartialOffset;
-    double *ms_part = pan_part + (int64_t)kMetricMaxCtas * kMetricStride;
+    double *ms_part = pan_part + kMetricRoom;
     int gp = 0, gm = 0, status_mask = 0;
     cudaError_t e;
     // PAN-resolution pass (unless the fused forward + metrics kernel wrote it)
@@ -1460,7 +1479,7 @@ cudaError_t launch_metrics(const MetricLaunch &m, cudaStream_t stream) {
         const FastFn fp = fast_fn(false, m.bands, m.a16 != 0);
         if (!m.a16) status_mask |= 1;
         const int64_t items = ((m.W + kStrip - 1) / kStrip) * ((m.H + kWin - 1) / kWin);
-        e = fast_grid(fp, items, &gp);
+        e = fast_grid(fp, items, m.bands, &gp);
         if (e != cudaSuccess) return e;
         a.partial = pan_part;
         void *args[] = {&a};
@@ -1469,7 +1488,7 @@ cudaError_t launch_metrics(const MetricLaunch &m, cudaStream_t stream) {
         const void *fp = m.fused_f32 ? (m.in_f32 ? pan_fn_nb<float, float>(m.bands) : pan_fn_nb<float, uint8_t>(m.bands))
                                      : (m.in_f32 ? pan_fn_nb<uint8_t, float>(m.bands) : pan_fn_nb<uint8_t, uint8_t>(m.bands));
         const int64_t items = ((m.W + kWarpCols - 1) / kWarpCols) * ((m.H + kWin - 1) / kWin);
-        e = grid_for(fp, items, &gp);
+        e = grid_for(fp, items, m.bands, &gp);
         if (e != cudaSuccess) return e;
         a.partial = pan_part;
         void *args[] = {&a};
@@ -1486,7 +1505,7 @@ cudaError_t launch_metrics(const MetricLaunch &m, cudaStream_t stream) {
         const FastFn fm = fast_fn(true, m.bands, m.a32_ms != 0);
         if (!m.a32_ms) status_mask |= 2;
         const int64_t items = ((m.W / 2 + kStrip - 1) / kStrip) * ((m.H / 2 + kWin - 1) / kWin);
-        e = fast_grid(fm, items, &gm, true);
+        e = fast_grid(fm, items, m.bands, &gm, true);
         if (e != cudaSuccess) return e;
         // The MS pass reads only MS and PAN.  When the kernel before it on the
     // stream is the PAN-resolution pass or the fused forward + metrics kernel
@@ -1508,7 +1527,7 @@ cudaError_t launch_metrics(const MetricLaunch &m, cudaStream_t stream) {
     } else {
         const void *fm = m.in_f32 ? ms_fn_nb<float>(m.bands) : ms_fn_nb<uint8_t>(m.bands);
         const int64_t items = ((m.W / 2 + kWarpCols - 1) / kWarpCols) * ((m.H / 2 + kWin - 1) / kWin);
-        e = grid_for(fm, items, &gm);
+        e = grid_for(fm, items, m.bands, &gm);
         if (e != cudaSuccess) return e;
         e = cudaLaunchKernel(fm, dim3(gm), dim3(kMThreads), args2, 0, stream);
     }
@@ -1518,9 +1537,9 @@ cudaError_t launch_metrics(const MetricLaunch &m, cudaStream_t stream) {
     const int fixed_mask = (m.pan_done || fast ? 1 : 0) | (m.in_f32 ? 0 : 2);
     double *result = m.result != out ? m.result : nullptr;
     const double *pp = pan_part, *mp = ms_part;
-    int nb = m.bands, want_q = m.want_q;
+    int stride = a.stride, nb = m.bands, want_q = m.want_q;
     int64_t H = m.H, W = m.W, nw_pan = nwp, nw_ms = nwm;
-    void *args3[] = {&pp, &mp, &gp, &gp_dev, &gm, &nb, &want_q, &H, &W, &nw_pan, &nw_ms, &status_mask,
+    void *args3[] = {&pp, &mp, &gp, &gp_dev, &gm, &stride, &nb, &want_q, &H, &W, &nw_pan, &nw_ms, &status_mask,
                      const_cast<int *>(&fixed_mask), &out, &result};
     // Programmatic dependent of the MS pass: its launch overlaps that pass's
     // end (it waits for the grid before it reads anything).
