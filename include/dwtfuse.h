@@ -186,7 +186,8 @@ int dwtfuse_fuse_backward(const float *grad_out, int bands, int64_t H, int64_t W
 size_t dwtfuse_metrics_workspace_size(void);
 
 /* Asynchronous on `stream`: writes four doubles to DEVICE memory out_device:
- * ERGAS, QNR, D_lambda, D_s.  Capturable in a CUDA graph.  On rows off the
+ * ERGAS, QNR, D_lambda, D_s (stored by the last kernel where it is memory of the
+ * launching device, else by a device-to-device copy).  Capturable in a CUDA graph.  On rows off the
  * 16-byte grid the passes wait on their own bulk copies; a wait that gives up
  * (about a second; not seen in normal operation) makes all four figures NaN,
  * and the synchronous dwtfuse_ergas / dwtfuse_qnr return DWTFUSE_ETIMEOUT. */

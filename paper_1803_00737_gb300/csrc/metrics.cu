@@ -1451,6 +1451,18 @@ cudaError_t grid_for(const void *fn, int64_t items, int bands, int *grid) {
     return cudaSuccess;
 }
 
+// Whether a kernel may store through p: memory of the launching device.  Another
+// GPU's memory needs peer access for that, and managed memory would move.
+bool on_this_device(const void *p) {
+    cudaPointerAttributes a;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();  // (the query's own error)
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 }  // namespace
 
 cudaError_t launch_metrics(const MetricLaunch &m, cudaStream_t stream) {
@@ -1535,7 +1547,10 @@ cudaError_t launch_metrics(const MetricLaunch &m, cudaStream_t stream) {
     const int64_t nwp = (m.H / kWin) * (m.W / kWin), nwm = (m.H / 2 / kWin) * (m.W / 2 / kWin);
     const int *gp_dev = m.pan_done ? reinterpret_cast<const int *>(m.workspace + kMetricPanCtasSlot) : nullptr;
     const int fixed_mask = (m.pan_done || fast ? 1 : 0) | (m.in_f32 ? 0 : 2);
-    double *result = m.result != out ? m.result : nullptr;
+    // The finalize stores the caller's figures itself where it can (a copy after
+    // it is one more node on the stream).
+    const bool wanted = m.result && m.result != out, direct = wanted && on_this_device(m.result);
+    double *result = direct ? m.result : nullptr;
     const double *pp = pan_part, *mp = ms_part;
     int stride = a.stride, nb = m.bands, want_q = m.want_q;
     int64_t H = m.H, W = m.W, nw_pan = nwp, nw_ms = nwm;
@@ -1552,7 +1567,10 @@ cudaError_t launch_metrics(const MetricLaunch &m, cudaStream_t stream) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(&metrics_finalize_kernel), args3);
+    e = cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(&metrics_finalize_kernel), args3);
+    if (e == cudaSuccess && wanted && !direct)
+        e = cudaMemcpyAsync(m.result, out, 4 * sizeof(double), cudaMemcpyDeviceToDevice, stream);
+    return e;
 }
 
 }  // namespace dwtfuse
