@@ -64,6 +64,8 @@ def fuse_batch_backward(g: torch.Tensor, wavelet: int, gp: torch.Tensor, gm: tor
     autotuner picked for this batch shape; a single scene through
     dwtfuse_fuse_backward."""
     N = g.shape[0]
+    if N == 0:
+        return
     if N == 1:
         _C.dwtfuse_fuse_backward(g[0], wavelet, gp[0], gm[0])
         return
