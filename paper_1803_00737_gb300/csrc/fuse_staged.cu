@@ -65,15 +65,13 @@ __device__ __forceinline__ void row_barrier() { asm volatile("barrier.sync 0;\n"
 template <bool SHIFT>
 constexpr int kStRow = kStCols + (SHIFT ? 8 : 0);
 
-template <int NB, bool SHIFT>
+template <int WAV, int NB, bool SHIFT, bool LATE>
 struct StagedEmit {
     static constexpr int kRow = kStRow<SHIFT>, kLay = SHIFT ? kShift : kVec;
     // Up to 4 bands: the next row's inputs loaded ahead (8192^2 x 3 208 -> 184
-    // us).  More: scalar synthesis, and the uint8 pixels stored after the
-    // float rows' copies are issued, behind the row barrier (16384^2 x 6 float
-    // + uint8 1388 -> 1340 us; with 3 bands that costs 208 -> 217).
-    static constexpr bool kLate = NB > 4;
-    static constexpr int kMode = NB > 4 ? kScalarCol | kScalarRow : kAheadPan | kAheadMs;
+    // us).  More: nothing ahead, D4 with scalar synthesis (its registers), Haar
+    // paired (loads ahead: 8190^2 x 6 uint8 to float 282 -> 306).
+    static constexpr int kMode = NB <= 4 ? kAheadPan | kAheadMs : WAV ? kScalarCol | kScalarRow : 0;
     const SceneArgs &s;
     const LaneCols &c;
     float *buf;    // two slots of [NB][2][kRow] floats
@@ -84,16 +82,16 @@ struct StagedEmit {
     int *rowc;     // the CTA's row count: row k fills slot k & 1
     bool hu;       // uint8 output wanted
     uint8_t *u;    // its band b0, the current MS row's first image row, column x
-    uint32_t w8[kLate ? NB : 1][2];  // kLate: the row's uint8 words
+    uint32_t w8[LATE ? NB : 1][2];  // LATE: the row's uint8 words
 
     __device__ __forceinline__ float *slot() const { return buf + (*rowc & 1) * (NB * 2 * kRow); }
 
     template <typename M>
     __device__ __forceinline__ void band(int b, const float *v0, const float *v1, M, M) {
-        if (kLate) {
+        if (LATE) {
             if (hu) {
-                w8[kLate ? b : 0][0] = pack4u8(v0);
-                w8[kLate ? b : 0][1] = pack4u8(v1);
+                w8[LATE ? b : 0][0] = pack4u8(v0);
+                w8[LATE ? b : 0][1] = pack4u8(v1);
             }
         } else {
             u += b ? s.out_plane : 0;
@@ -108,7 +106,7 @@ struct StagedEmit {
                 *reinterpret_cast<float4 *>(row + kRow) = make_float4(v1[0], v1[1], v1[2], v1[3]);
             }
         }
-        if (!kLate && hu) store_rows(u, pack4u8(v0), pack4u8(v1));
+        if (!LATE && hu) store_rows(u, pack4u8(v0), pack4u8(v1));
     }
 
     __device__ __forceinline__ void store_rows(uint8_t *q, uint32_t w0, uint32_t w1) const {
@@ -146,11 +144,11 @@ struct StagedEmit {
             }
             asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
         }
-        if (kLate) {
+        if (LATE) {
             if (hu) {
                 uint8_t *q = u;
 #pragma unroll
-                for (int b = 0; b < (kLate ? NB : 1); ++b) {
+                for (int b = 0; b < (LATE ? NB : 1); ++b) {
                     store_rows(q, w8[b][0], w8[b][1]);
                     q += s.out_plane;
                 }
@@ -165,7 +163,7 @@ struct StagedEmit {
 
 // One CTA item: columns [X0, X0 + 1024), MS rows [m_s, m_e), bands
 // [b0, b0 + NB).  Every thread of the CTA calls it, with the same row count.
-template <typename T, int WAV, int NB, bool SHIFT>
+template <typename T, int WAV, int NB, bool SHIFT, bool LATE>
 __device__ __forceinline__ void staged_item(const SceneArgs &s, float *buf, int64_t X0, int m_s, int m_e, int b0,
                                             int *rowc) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -173,7 +171,7 @@ __device__ __forceinline__ void staged_item(const SceneArgs &s, float *buf, int6
     const LaneCols c = lane_cols(x0, lane, s.W);  // warps past W: idle lanes
     const int ncols = (int)min((int64_t)kStCols, s.W - X0);
     uint8_t *u = s.out_u8 + (int64_t)b0 * s.out_plane + (int64_t)(2 * (m_s - s.m_lo)) * s.W + c.x;
-    StagedEmit<NB, SHIFT> out{s, c, buf, X0, ncols, lane, b0, rowc, s.out_u8 != nullptr, u};
+    StagedEmit<WAV, NB, SHIFT, LATE> out{s, c, buf, X0, ncols, lane, b0, rowc, s.out_u8 != nullptr, u};
     walk_rows<T, WAV, NB, SHIFT ? kShift : kVec>(s, c, x0, m_s, m_e, b0, out);
 }
 
@@ -184,7 +182,7 @@ __device__ __forceinline__ void bulk_drain() {
 }  // namespace
 
 // Single scene, bands [b0, b0 + NB); CTA items it = blockIdx.x, + gridDim.x, ...
-template <typename T, int WAV, int NB, bool SHIFT>
+template <typename T, int WAV, int NB, bool SHIFT, bool LATE>
 __global__ void __launch_bounds__(kStThreads, 2)
 fuse_staged_kernel(const __grid_constant__ SceneArgs s, int b0, int64_t strips_cta, int64_t items, int R) {
     extern __shared__ __align__(128) float st_buf[];
@@ -192,7 +190,7 @@ fuse_staged_kernel(const __grid_constant__ SceneArgs s, int b0, int64_t strips_c
     for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
         const int64_t sx = it % strips_cta, sy = it / strips_cta;
         const int m_s = s.m_lo + (int)(sy * R);
-        staged_item<T, WAV, NB, SHIFT>(s, st_buf, sx * kStCols, m_s, min(m_s + R, s.m_hi), b0, &rowc);
+        staged_item<T, WAV, NB, SHIFT, LATE>(s, st_buf, sx * kStCols, m_s, min(m_s + R, s.m_hi), b0, &rowc);
     }
     bulk_drain();
 }
@@ -200,20 +198,22 @@ fuse_staged_kernel(const __grid_constant__ SceneArgs s, int b0, int64_t strips_c
 namespace {
 
 template <typename T, int WAV, int NB>
-void *st_fn_nb(bool shift) {
-    return shift ? reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, NB, true>)
-                 : reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, NB, false>);
+void *st_fn_nb(bool shift, bool late) {
+    if constexpr (NB == 6 && (WAV || sizeof(T) == 1))
+        if (late) return reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, NB, false, true>);
+    return shift ? reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, NB, true, false>)
+                 : reinterpret_cast<void *>(&fuse_staged_kernel<T, WAV, NB, false, false>);
 }
 
 template <typename T, int WAV>
-void *st_fn(int nb, bool shift) {
+void *st_fn(int nb, bool shift, bool late) {
     switch (nb) {
-        case 1: return st_fn_nb<T, WAV, 1>(shift);
-        case 2: return st_fn_nb<T, WAV, 2>(shift);
-        case 3: return st_fn_nb<T, WAV, 3>(shift);
-        case 4: return st_fn_nb<T, WAV, 4>(shift);
-        case 5: return st_fn_nb<T, WAV, 5>(shift);
-        case 6: return st_fn_nb<T, WAV, 6>(shift);
+        case 1: return st_fn_nb<T, WAV, 1>(shift, late);
+        case 2: return st_fn_nb<T, WAV, 2>(shift, late);
+        case 3: return st_fn_nb<T, WAV, 3>(shift, late);
+        case 4: return st_fn_nb<T, WAV, 4>(shift, late);
+        case 5: return st_fn_nb<T, WAV, 5>(shift, late);
+        case 6: return st_fn_nb<T, WAV, 6>(shift, late);
         default: return nullptr;
     }
 }
@@ -254,6 +254,18 @@ bool fuse_staged_applies(const SceneArgs &s) {
     return (strips * kStCols - s.W) * 8 <= strips * kStCols;
 }
 
+// Whether the uint8 pixels are stored after the float rows' copies are issued,
+// behind the row barrier, instead of band by band before it.  Only 6 bands on
+// aligned rows gain by it, and not all of them.  us, before -> behind, float +
+// uint8: D4 on the 128-byte line grid 16384^2 1378 -> 1334, 8192^2 347 -> 337;
+// off that grid uint8 3000 x 4092 69.7 -> 70.5, float 82.8 -> 85.5, 4958 x 7932
+// 258 -> 263; Haar uint8 8192^2 365 -> 353, 4958 x 7932 229 -> 214; Haar float
+// 4958 x 7932 262 -> 280.  Five bands lose (D4 4096^2 76.2 -> 80.0, 12000 x 12284
+// 645 -> 687), and so do shifted rows (8190^2 x 6 356 -> 389).
+static bool staged_late(const SceneArgs &s, int nb) {
+    return nb == 6 && s.a4 != 0 && s.out_u8 != nullptr && (s.wavelet ? s.W % 32 == 0 : s.in_f32 == 0);
+}
+
 static int64_t staged_strips(int64_t W) { return (W + kStCols - 1) / kStCols; }
 
 cudaError_t launch_fuse_staged(const SceneArgs &s, int R, cudaStream_t stream) {
@@ -268,8 +280,9 @@ cudaError_t launch_fuse_staged(const SceneArgs &s, int R, cudaStream_t stream) {
     for (int b0 = 0; b0 < s.bands; b0 += chunk) {
         const int nb = s.bands - b0 < chunk ? s.bands - b0 : chunk;
         const bool shift = s.a4 == 0;
-        void *fn = s.in_f32 ? (s.wavelet ? st_fn<float, 1>(nb, shift) : st_fn<float, 0>(nb, shift))
-                            : (s.wavelet ? st_fn<uint8_t, 1>(nb, shift) : st_fn<uint8_t, 0>(nb, shift));
+        const bool late = staged_late(s, nb);
+        void *fn = s.in_f32 ? (s.wavelet ? st_fn<float, 1>(nb, shift, late) : st_fn<float, 0>(nb, shift, late))
+                            : (s.wavelet ? st_fn<uint8_t, 1>(nb, shift, late) : st_fn<uint8_t, 0>(nb, shift, late));
         if (fn == nullptr) return cudaErrorInvalidValue;
         const int smem = staged_smem(nb, shift);
         int occ = 0;
