@@ -16,17 +16,20 @@ constexpr int kShiftRows = 4;
 // an instance.  With a float output: up to 4 bands PAN one row ahead (3736 x
 // 4070 x 3 uint8 58 -> 53.5); more bands scalar columns (8192^2 x 8 uint8 to
 // float + uint8 502 -> 491), floats scalar rows too (8192^2 x 8 522 -> 493, 6
-// bands on shifted rows 405 -> 398).  A uint8 output alone leaves the walker
+// bands on shifted rows 405 -> 398), Haar, whose walker keeps no synthesised
+// row, everything ahead (floats to float + uint8, 3000 x 3002 x 5 64 -> 58, 4000
+// x 4002 x 6 130 -> 124; uint8 106 -> 101).  A uint8 output alone leaves the walker
 // bound by instructions and load latency: paired FP32 and loads ahead as far as
 // the registers go, at 8192^2: 3 bands 109 -> 103, 5 bands 155 -> 134, 7 bands
 // 191 -> 175; 8 bands with 12 warps per SM whose registers hold the next row's
 // inputs (208 -> 194; 7480 x 8140 193 -> 174).
-template <typename T, int NB, bool U8ONLY>
+template <typename T, int WAV, int NB, bool U8ONLY>
 struct FwdShape {
     static constexpr int kThreads = U8ONLY && NB == 8 ? 192 : 256;
     static constexpr int kWarps = kThreads / 32;
     static constexpr int kMode = U8ONLY    ? (NB <= 4 || NB == 8 ? kAheadPan | kAheadMs : NB <= 6 ? kAheadPan : 0)
                                  : NB <= 4 ? kAheadPan
+                                 : WAV == 0 ? kAheadPan | kAheadMs
                                            : (sizeof(T) == 4 ? kScalarCol | kScalarRow : kScalarCol);
     // (8 bands: the walker without its float stores compiled to a slower
     // schedule, 193 us against 174, so that instance keeps the run-time test)
@@ -38,9 +41,9 @@ struct FwdShape {
 // Row layout: SHIFT kShift, else VEC kVec, else kPairs.  U8ONLY: a uint8
 // output and no float one.
 template <typename T, int WAV, int NB, bool U8ONLY, bool VEC, bool SHIFT>
-__global__ void __launch_bounds__(FwdShape<T, NB, U8ONLY>::kThreads, 2)
+__global__ void __launch_bounds__(FwdShape<T, WAV, NB, U8ONLY>::kThreads, 2)
 fuse_fwd_kernel(const __grid_constant__ SceneArgs s, int b0, int64_t strips_x, int64_t items, int R) {
-    using F = FwdShape<T, NB, U8ONLY>;
+    using F = FwdShape<T, WAV, NB, U8ONLY>;
     constexpr int LAY = SHIFT ? kShift : (VEC ? kVec : kPairs);
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t)gridDim.x * F::kWarps;
@@ -59,7 +62,7 @@ struct FwdFn {
 
 template <typename T, int WAV, int NB, bool U8ONLY>
 FwdFn fwd_fn(int lay) {
-    constexpr int kT = FwdShape<T, NB, U8ONLY>::kThreads;
+    constexpr int kT = FwdShape<T, WAV, NB, U8ONLY>::kThreads;
     if (lay == kVec) return {reinterpret_cast<void *>(&fuse_fwd_kernel<T, WAV, NB, U8ONLY, true, false>), kT};
     if constexpr (NB <= kAltMaxBands)
         if (lay == kShift) return {reinterpret_cast<void *>(&fuse_fwd_kernel<T, WAV, NB, U8ONLY, false, true>), kT};
