@@ -235,7 +235,11 @@ constexpr int staged_smem(int nb, bool shift) {
 // -> 197, 8192 x 8140 x 8 554 -> 504, 16384^2 x 8 1952 -> 1910, 8192^2 x 12 733
 // -> 675; below the line 3736 x 4070 x 3 47 -> 51, 3000 x 2998 x 5 48 -> 55,
 // 4096^2 x 8 float 102 -> 107.  Float scenes of more than 6 aligned bands read
-// four times the PAN bytes per chunk and stay on the warp kernel.  The same CTA
+// four times the PAN bytes per chunk and stay on the warp kernel; so do, for
+// float alone, the 7 and 8 aligned bands that D4 takes in one warp launch, 8 up to
+// four times that line (staged -> warp: 8192^2 x 7 349 -> 335, 16384^2 x 7 1362 ->
+// 1333, 4096 x 8192 x 8 197 -> 194, 8192^2 x 8 381 -> 378; 12000 x 12288 x 8 827 ->
+// 830, 16384^2 x 8 1491 -> 1515; Haar 8192^2 x 7 339 -> 350).  The same CTA
 // items in the batched launch ran slower than its warp items on every scene
 // class tried (46 scenes on the grid: 5356 -> 4651 GB/s; with the next item
 // fetched during the current one and 64-row items: 4644), so the batched
@@ -247,8 +251,11 @@ bool fuse_staged_applies(const SceneArgs &s) {
     const bool more = s.bands > kStagedMaxBands;
     if (s.a4 == 0 || more) {
         if (s.a4 != 0 && s.in_f32) return false;
-        const int64_t px = 2 * (int64_t)(s.m_hi - s.m_lo) * s.W * s.bands;
-        if (px * (s.out_u8 ? 5 : 4) < kStagedLarge) return false;
+        const int64_t px = 2 * (int64_t)(s.m_hi - s.m_lo) * s.W * s.bands, bytes = px * (s.out_u8 ? 5 : 4);
+        if (bytes < kStagedLarge) return false;
+        if (s.a4 != 0 && s.wavelet && s.out_u8 == nullptr &&
+            (s.bands < kChunkBands || (s.bands == kChunkBands && bytes < 4 * kStagedLarge)))
+            return false;
     }
     const int64_t strips = (s.W + kStCols - 1) / kStCols;
     return (strips * kStCols - s.W) * 8 <= strips * kStCols;
