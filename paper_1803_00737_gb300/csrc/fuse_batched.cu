@@ -142,63 +142,79 @@ cudaError_t launch_table(const BatchTable &t, unsigned long long *queue, int *st
     return cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, (size_t)smem, stream);
 }
 
-// MS rows per item of a launch over entries order[0 .. m): a tenth of a warp's
+// MS rows per item of a launch over table t: a tenth of a warp's
 // share of the rows (16 warps per SM), at most kDefaultRows, so that the
 // queue's last items leave little of the GPU idle (24 uneven scenes, 94 and 75
 // rows a warp in the two launches: 32 rows 721 us a call, 16 rows 653, 8 rows
 // 644), and down to single rows, so that small tables still reach every warp
 // (8 scenes of 256..600 px: 106 -> 40 us); large uniform tables keep tall
 // items (8 x 4096^2 x 4 float, 215 rows a warp: 24 rows 521 us, 8 rows 533).
-int default_rows(const BatchTable &t, const int *order, int m, int sms) {
+int default_rows(const BatchTable &t, int sms) {
     double rows = 0;
-    for (int j = 0; j < m; ++j)
-        rows += (double)t.strips_x[order[j]] * (t.scenes[order[j]].m_hi - t.scenes[order[j]].m_lo);
+    for (int i = 0; i < t.n; ++i) rows += (double)t.strips_x[i] * (t.scenes[i].m_hi - t.scenes[i].m_lo);
     const double share = rows / (16.0 * sms), low = share < 4 ? share : 4;
     const double r = share / 10 > low ? share / 10 : low;
     return r < 1 ? 1 : (r > kDefaultRows ? kDefaultRows : (int)(r + 0.5));
 }
 
+// Bands, wavelet and row layout of an entry: the item body it runs.
+int body_of(const SceneArgs &s) { return (s.bands * 2 + s.wavelet) * 3 + row_layout(s.a4, s.alt); }
+
 // The entries of t of input type f32 and width class narrow (at most
-// kBatchNarrowBands bands or more), those of one body (bands, wavelet, row
-// layout) together: warps of an SM work on neighbouring items, so they run one
-// or two bodies at a time and share their instructions (24 uneven scenes in
-// the caller's order: 768 us, instruction fetch 1.9 of 12 stall cycles per
-// issue; sorted 719 us).
-void split_table(const BatchTable &t, bool f32, bool narrow, int sms, BatchTable *o) {
+// kBatchNarrowBands bands or more), those of one body together: warps of an SM
+// work on neighbouring items, so they run one or two bodies at a time and share
+// their instructions (24 uneven scenes in the caller's order: 768 us,
+// instruction fetch 1.9 of 12 stall cycles per issue; sorted 719 us).
+void split_table(const BatchTable &t, bool f32, bool narrow, BatchTable *o) {
     int order[kMaxScenes], m = 0;
     for (int i = 0; i < t.n; ++i)
         if ((t.scenes[i].in_f32 != 0) == f32 && (t.scenes[i].bands <= kBatchNarrowBands) == narrow) order[m++] = i;
-    auto body = [&](int i) {
-        return (t.scenes[i].bands * 2 + t.scenes[i].wavelet) * 3 + row_layout(t.scenes[i].a4, t.scenes[i].alt);
-    };
-    std::stable_sort(order, order + m, [&](int a, int b) { return body(a) > body(b); });
+    std::stable_sort(order, order + m, [&](int a, int b) { return body_of(t.scenes[a]) > body_of(t.scenes[b]); });
     o->n = m;
-    o->R = t.R > 0 ? t.R : default_rows(t, order, m, sms);
-    o->item_start[0] = 0;
+    o->R = t.R;
     for (int j = 0; j < m; ++j) {
-        const SceneArgs &s = t.scenes[order[j]];
-        o->scenes[j] = s;
+        o->scenes[j] = t.scenes[order[j]];
         o->strips_x[j] = t.strips_x[order[j]];
-        o->item_start[j + 1] = o->item_start[j] + o->strips_x[j] * ((s.m_hi - s.m_lo + o->R - 1) / o->R);
+    }
+}
+
+// Item height (where the caller left it open) and item ranges of a launch's table.
+void lay_out_items(BatchTable *t, int sms) {
+    if (t->R <= 0) t->R = default_rows(*t, sms);
+    t->item_start[0] = 0;
+    for (int j = 0; j < t->n; ++j) {
+        const SceneArgs &s = t->scenes[j];
+        t->item_start[j + 1] = t->item_start[j] + t->strips_x[j] * ((s.m_hi - s.m_lo + t->R - 1) / t->R);
     }
 }
 
 }  // namespace
 
 // One launch per input type and width class in the table, the wide ones first.
-cudaError_t launch_fuse_batched(const BatchTable &t, unsigned long long *queue, int *status,
+// A table of one body (a batch tensor) is launched as it is: copying its
+// entries cost 4 us of a call (128 scenes of 128^2 x 3: 41 -> 45 us).
+cudaError_t launch_fuse_batched(BatchTable &t, unsigned long long *queue, int *status,
                                 int blocks_per_sm, cudaStream_t stream) {
     int count[2][2] = {};
-    for (int i = 0; i < t.n; ++i) ++count[t.scenes[i].in_f32 != 0][t.scenes[i].bands <= kBatchNarrowBands];
-    static thread_local BatchTable part;
+    bool one_body = true;
+    for (int i = 0; i < t.n; ++i) {
+        ++count[t.scenes[i].in_f32 != 0][t.scenes[i].bands <= kBatchNarrowBands];
+        one_body = one_body && t.scenes[i].in_f32 == t.scenes[0].in_f32 && body_of(t.scenes[i]) == body_of(t.scenes[0]);
+    }
     int sms = 0;
     const cudaError_t es = sm_count(&sms);
     if (es != cudaSuccess) return es;
+    if (one_body && t.n > 0) {
+        lay_out_items(&t, sms);
+        return launch_table(t, queue, status, blocks_per_sm, kQueueBytes, stream);
+    }
+    static thread_local BatchTable part;
     size_t clear = kQueueBytes;
     for (int kind = 0; kind < 4; ++kind) {
         const bool narrow = kind >> 1, f32 = kind & 1;
         if (count[f32][narrow] == 0) continue;
-        split_table(t, f32, narrow, sms, &part);
+        split_table(t, f32, narrow, &part);
+        lay_out_items(&part, sms);
         const cudaError_t e = launch_table(part, queue, status, blocks_per_sm, clear, stream);
         if (e != cudaSuccess) return e;
         clear = sizeof(unsigned long long);

@@ -136,7 +136,7 @@ cudaError_t launch_fuse_metrics(const SceneArgs &s, double *pan_partial, int str
 constexpr int64_t kMetricPanCtasSlot = 4;
 constexpr int64_t kMetricStatusSlot = 5;  // int: DWTFUSE_OK, or DWTFUSE_ETIMEOUT when a bounded wait gave up
 constexpr int64_t kMetricPanPartialOffset = 8;
-cudaError_t launch_fuse_batched(const BatchTable &t, unsigned long long *queue, int *status,
+cudaError_t launch_fuse_batched(BatchTable &t, unsigned long long *queue, int *status,
                                 int blocks_per_sm, cudaStream_t stream);
 
 // Staged single-scene forward (fuse_staged.cu): taken for rows on the 16-byte
