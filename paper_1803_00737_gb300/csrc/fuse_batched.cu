@@ -26,6 +26,7 @@ struct BatchShape {
     static constexpr int kMode = kNarrow ? (kFloat ? kAheadPan | kAheadMs : 0)
                                          : (kFloat ? kScalarCol | kScalarRow : kAheadPan);
     static constexpr int kSmem = kThreads / 32 * kSceneBytes;
+    static constexpr int kMinBands = kNarrow ? 1 : kBatchNarrowBands + 1;  // fewer: the narrow instance's entries
 };
 
 extern __shared__ __align__(16) unsigned char batch_smem[];
@@ -39,6 +40,23 @@ template <typename T, int WAV, int NB, int LAY, int MODE>
 static __device__ __noinline__ void batch_body(int x0, int m_s, int m_e) {
     const SceneArgs &s = *reinterpret_cast<const SceneArgs *>(batch_smem + (threadIdx.x >> 5) * kSceneBytes);
     direct_item<T, WAV, NB, LAY, MODE>(s, x0, m_s, m_e, 0, threadIdx.x & 31);
+}
+
+// The item by its entry's row layout (entries on shifted rows hold at most
+// kBatchAltMaxBands bands: the table splits them or clears alt).
+template <typename T, int WAV, int NB, int MODE>
+static __device__ __forceinline__ void batch_item(const SceneArgs &s, int x0, int m_s, int m_e) {
+    if (s.a4) {
+        batch_body<T, WAV, NB, kVec, MODE>(x0, m_s, m_e);
+        return;
+    }
+    if constexpr (NB <= kBatchAltMaxBands) {
+        if (s.alt) {
+            batch_body<T, WAV, NB, kShift, MODE>(x0, m_s, m_e);
+            return;
+        }
+    }
+    batch_body<T, WAV, NB, kPairs, MODE>(x0, m_s, m_e);
 }
 
 // Batched: every warp pulls the next item index from `queue[0]`; item ranges
@@ -64,7 +82,7 @@ fuse_batched_kernel(const __grid_constant__ BatchTable t, unsigned long long *qu
             if ((unsigned long long)t.item_start[mid] <= it) lo = mid; else hi = mid - 1;
         }
         const SceneArgs &s = t.scenes[lo];
-        if (s.bands < 1 || s.bands > MAXB || (s.in_f32 != 0) != (sizeof(T) == 4)) {
+        if (s.bands < BatchShape<T, MAXB>::kMinBands || s.bands > MAXB || (s.in_f32 != 0) != (sizeof(T) == 4)) {
             if (lane == 0) atomicCAS(status, 0, 7);
             continue;
         }
@@ -80,16 +98,9 @@ fuse_batched_kernel(const __grid_constant__ BatchTable t, unsigned long long *qu
         const int x0 = (int)(sx * kWarpCols), m_s = s.m_lo + (int)(sy * t.R), m_e = min(m_s + t.R, s.m_hi);
 #define DWTFUSE_CASE(NBV)                                                      \
     case NBV:                                                                  \
-        if constexpr (NBV <= MAXB) {                                           \
-            if (s.wavelet) {                                                   \
-                if (s.a4) batch_body<T, 1, NBV, kVec, M>(x0, m_s, m_e);           \
-                else if (s.alt) batch_body<T, 1, NBV, kShift, M>(x0, m_s, m_e);   \
-                else batch_body<T, 1, NBV, kPairs, M>(x0, m_s, m_e);              \
-            } else {                                                           \
-                if (s.a4) batch_body<T, 0, NBV, kVec, M>(x0, m_s, m_e);           \
-                else if (s.alt) batch_body<T, 0, NBV, kShift, M>(x0, m_s, m_e);   \
-                else batch_body<T, 0, NBV, kPairs, M>(x0, m_s, m_e);              \
-            }                                                                  \
+        if constexpr (NBV >= BatchShape<T, MAXB>::kMinBands && NBV <= MAXB) {  \
+            if (s.wavelet) batch_item<T, 1, NBV, M>(s, x0, m_s, m_e);          \
+            else batch_item<T, 0, NBV, M>(s, x0, m_s, m_e);                    \
         }                                                                      \
         break;
         switch (s.bands) {

@@ -97,8 +97,6 @@ __device__ __forceinline__ void ld4(const float *p, float *v) {
     v[2] = q.z;
     v[3] = q.w;
 }
-__device__ __forceinline__ float ld1(const uint8_t *p) { return (float)__ldg(p); }
-__device__ __forceinline__ float ld1(const float *p) { return __ldg(p); }
 
 // ------------------------------------------------------------------ stores
 
