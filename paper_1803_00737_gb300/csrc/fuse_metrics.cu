@@ -95,7 +95,9 @@ template <int NB, int LAY>
 struct MetricEmit {
     using L = FmLayout<NB>;
     static constexpr bool kAllLanes = true;
-    static constexpr int kMode = kScalarCol;
+    // Paired row synthesis but for 7 bands, whose D4 walker spills with it (144
+    // bytes on aligned rows: 8192^2 733 -> 531 us, 8190^2 675 -> 659).
+    static constexpr int kMode = NB == 7 ? kScalarCol | kScalarRow : kScalarCol;
     static constexpr int K = L::K, P = L::P, NS = L::NS, SR = L::SR;
     const SceneArgs &s;
     const LaneCols &c;
