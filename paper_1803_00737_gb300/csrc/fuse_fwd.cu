@@ -9,7 +9,9 @@ constexpr int kAltMaxBands = 6;  // widest band chunk of the shifted-row instanc
 // items bring them there close together (rows per item 4 against the balanced
 // height: 16384 x 16382 x 6 float + uint8 1948 -> 1804 us, 5000 x 5002 x 6 174
 // -> 160, 3736 x 4070 x 3 49.2 -> 46.2; aligned rows gain nothing: 8192^2 x 8
-// float 520 -> 526).
+// float 520 -> 526).  Not for one or two bands of floats to uint8 alone, which
+// read more than they write (8190^2 D4, short -> balanced: one band 125 -> 105,
+// two 150 -> 127; Haar, one 81 -> 75).
 constexpr int kShiftRows = 4;
 
 // Walker mode (paired / scalar FP32 and loads ahead, us a call) and CTA size of
@@ -126,7 +128,10 @@ cudaError_t launch_fuse(const SceneArgs &s, int R, int blocks_per_sm, cudaStream
         int Rl = R;
         if (Rl <= 0) {
             Rl = balanced_rows((s.W + kWarpCols - 1) / kWarpCols, rows2 / 2, cap * warps);
-            if (alt && Rl > kShiftRows) Rl = kShiftRows;
+            // (the least output bytes a pixel for which they pay, against the PAN bytes that
+            // short items read again)
+            const int px_out = nb * ((s.out_f32 ? 4 : 0) + (s.out_u8 ? 1 : 0)), px_pan = s.in_f32 ? 4 : 1;
+            if (alt && 2 * px_out > px_pan && Rl > kShiftRows) Rl = kShiftRows;
         }
         const ItemGrid g = item_grid(rows2, s.W, Rl);
         const int64_t need = (g.items + warps - 1) / warps;
