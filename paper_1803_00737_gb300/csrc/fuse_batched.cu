@@ -17,14 +17,17 @@ constexpr int kSceneBytes = (int)((sizeof(SceneArgs) + 15) / 16 * 16);
 // 8 x 4096^2 x 4: 1086 us a pass against 1129 with 20 warps, where that
 // spills, and 1101 with 16 and no loads ahead).  More bands, 16 warps: floats
 // with scalar synthesis (4 x 4096^2 x 8 570 -> 480 us a call, 8 x 2048^2 x 8
-// 298 -> 248; paired, the walker spills), uint8 paired with PAN ahead (24
-// uneven scenes to uint8 469 -> 464).
+// 298 -> 248; paired, the walker spills more), uint8 paired with PAN ahead (24
+// uneven scenes to uint8 469 -> 464) but for 8 bands of D4, which then spill 212
+// bytes a thread (to float 4 x 4096^2 430 -> 377, 16 x 1000 x 1004 120 -> 108).
 template <typename T, int MAXB>
 struct BatchShape {
     static constexpr bool kNarrow = MAXB <= kBatchNarrowBands, kFloat = sizeof(T) == 4;
     static constexpr int kThreads = kNarrow && !kFloat ? 320 : 256;
-    static constexpr int kMode = kNarrow ? (kFloat ? kAheadPan | kAheadMs : 0)
-                                         : (kFloat ? kScalarCol | kScalarRow : kAheadPan);
+    template <int WAV, int NB>
+    static constexpr int kMode = kNarrow  ? (kFloat ? kAheadPan | kAheadMs : 0)
+                                 : kFloat ? kScalarCol | kScalarRow
+                                          : (WAV && NB == 8 ? kScalarCol : kAheadPan);
     static constexpr int kSmem = kThreads / 32 * kSceneBytes;
     static constexpr int kMinBands = kNarrow ? 1 : kBatchNarrowBands + 1;  // fewer: the narrow instance's entries
 };
@@ -66,7 +69,6 @@ static __device__ __forceinline__ void batch_item(const SceneArgs &s, int x0, in
 template <typename T, int MAXB>
 __global__ void __launch_bounds__(BatchShape<T, MAXB>::kThreads, 2)
 fuse_batched_kernel(const __grid_constant__ BatchTable t, unsigned long long *queue, int *status) {
-    constexpr int M = BatchShape<T, MAXB>::kMode;
     uint32_t *copy = reinterpret_cast<uint32_t *>(batch_smem + (threadIdx.x >> 5) * kSceneBytes);
     const int lane = threadIdx.x & 31;
     const unsigned long long total = (unsigned long long)t.item_start[t.n];
@@ -82,7 +84,8 @@ fuse_batched_kernel(const __grid_constant__ BatchTable t, unsigned long long *qu
             if ((unsigned long long)t.item_start[mid] <= it) lo = mid; else hi = mid - 1;
         }
         const SceneArgs &s = t.scenes[lo];
-        if (s.bands < BatchShape<T, MAXB>::kMinBands || s.bands > MAXB || (s.in_f32 != 0) != (sizeof(T) == 4)) {
+        using Shape = BatchShape<T, MAXB>;
+        if (s.bands < Shape::kMinBands || s.bands > MAXB || (s.in_f32 != 0) != (sizeof(T) == 4)) {
             if (lane == 0) atomicCAS(status, 0, 7);
             continue;
         }
@@ -96,12 +99,15 @@ fuse_batched_kernel(const __grid_constant__ BatchTable t, unsigned long long *qu
         const int64_t local = (int64_t)(it - (unsigned long long)t.item_start[lo]);
         const int64_t sx = local % t.strips_x[lo], sy = local / t.strips_x[lo];
         const int x0 = (int)(sx * kWarpCols), m_s = s.m_lo + (int)(sy * t.R), m_e = min(m_s + t.R, s.m_hi);
-#define DWTFUSE_CASE(NBV)                                                      \
-    case NBV:                                                                  \
-        if constexpr (NBV >= BatchShape<T, MAXB>::kMinBands && NBV <= MAXB) {  \
-            if (s.wavelet) batch_item<T, 1, NBV, M>(s, x0, m_s, m_e);          \
-            else batch_item<T, 0, NBV, M>(s, x0, m_s, m_e);                    \
-        }                                                                      \
+#define DWTFUSE_CASE(NBV)                                                                        \
+    case NBV:                                                                                    \
+        if constexpr (NBV >= Shape::kMinBands && NBV <= MAXB) {                                  \
+            if (!s.wavelet) {                                                                    \
+                batch_item<T, 0, NBV, Shape::template kMode<0, NBV>>(s, x0, m_s, m_e);           \
+            } else {                                                                           \
+                batch_item<T, 1, NBV, Shape::template kMode<1, NBV>>(s, x0, m_s, m_e);           \
+            }                                                                                    \
+        }                                                                                        \
         break;
         switch (s.bands) {
             DWTFUSE_CASE(1) DWTFUSE_CASE(2) DWTFUSE_CASE(3) DWTFUSE_CASE(4)
