@@ -7,6 +7,11 @@
 namespace dwtfuse {
 
 constexpr int kBatchNarrowBands = 4;  // instance for entries of at most 4 bands
+constexpr int kBatchLightBands = 3;   // float instance for entries of light bodies alone
+// A float body whose registers leave room for 20 warps per SM.
+__host__ __device__ constexpr bool light_body(int wavelet, int bands) {
+    return bands == 1 || (wavelet == 0 && bands <= kBatchLightBands);
+}
 constexpr int kSceneBytes = (int)((sizeof(SceneArgs) + 15) / 16 * 16);
 
 // Threads per CTA (two CTAs per SM), walker mode and shared memory (per warp, a
@@ -15,7 +20,10 @@ constexpr int kSceneBytes = (int)((sizeof(SceneArgs) + 15) / 16 * 16);
 // 256..4096 px: 719 us a call against 730 with 16 warps at 128), float 16
 // warps with the next row's inputs loaded ahead (forward + backward of
 // 8 x 4096^2 x 4: 1086 us a pass against 1129 with 20 warps, where that
-// spills, and 1101 with 16 and no loads ahead).  More bands, 16 warps: floats
+// spills, and 1101 with 16 and no loads ahead), or 20 warps where all entries are
+// Haar of at most 3 bands or have one band (4 x 4096^2, 16 -> 20 warps: Haar x 1 125
+// -> 116, x 2 170 -> 159, x 3 213 -> 202, D4 x 1 134 -> 122; D4 x 2 and x 3 spill
+// there, 181 -> 202, 237 -> 284).  More bands, 16 warps: floats
 // with scalar synthesis (4 x 4096^2 x 8 570 -> 480 us a call, 8 x 2048^2 x 8
 // 298 -> 248; paired, the walker spills more), uint8 paired with PAN ahead (24
 // uneven scenes to uint8 469 -> 464) but for 8 bands of D4, which then spill 212
@@ -23,7 +31,8 @@ constexpr int kSceneBytes = (int)((sizeof(SceneArgs) + 15) / 16 * 16);
 template <typename T, int MAXB>
 struct BatchShape {
     static constexpr bool kNarrow = MAXB <= kBatchNarrowBands, kFloat = sizeof(T) == 4;
-    static constexpr int kThreads = kNarrow && !kFloat ? 320 : 256;
+    static constexpr bool kLight = kFloat && MAXB == kBatchLightBands;
+    static constexpr int kThreads = kNarrow && (!kFloat || kLight) ? 320 : 256;
     template <int WAV, int NB>
     static constexpr int kMode = kNarrow  ? (kFloat ? kAheadPan | kAheadMs : 0)
                                  : kFloat ? kScalarCol | kScalarRow
@@ -85,7 +94,8 @@ fuse_batched_kernel(const __grid_constant__ BatchTable t, unsigned long long *qu
         }
         const SceneArgs &s = t.scenes[lo];
         using Shape = BatchShape<T, MAXB>;
-        if (s.bands < Shape::kMinBands || s.bands > MAXB || (s.in_f32 != 0) != (sizeof(T) == 4)) {
+        if (s.bands < Shape::kMinBands || s.bands > MAXB || (s.in_f32 != 0) != (sizeof(T) == 4) ||
+            (Shape::kLight && !light_body(s.wavelet, s.bands))) {
             if (lane == 0) atomicCAS(status, 0, 7);
             continue;
         }
@@ -104,7 +114,7 @@ fuse_batched_kernel(const __grid_constant__ BatchTable t, unsigned long long *qu
         if constexpr (NBV >= Shape::kMinBands && NBV <= MAXB) {                                  \
             if (!s.wavelet) {                                                                    \
                 batch_item<T, 0, NBV, Shape::template kMode<0, NBV>>(s, x0, m_s, m_e);           \
-            } else {                                                                           \
+            } else if constexpr (!Shape::kLight || light_body(1, NBV)) {                         \
                 batch_item<T, 1, NBV, Shape::template kMode<1, NBV>>(s, x0, m_s, m_e);           \
             }                                                                                    \
         }                                                                                        \
@@ -137,8 +147,11 @@ BatchFn batch_fn() {
 cudaError_t launch_table(const BatchTable &t, unsigned long long *queue, int *status, int blocks_per_sm,
                          size_t clear, cudaStream_t stream) {
     const bool f32 = t.scenes[0].in_f32 != 0, narrow = t.scenes[0].bands <= kBatchNarrowBands;
-    const BatchFn k = f32 ? (narrow ? batch_fn<float, kBatchNarrowBands>() : batch_fn<float, kBatchMaxBands>())
-                          : (narrow ? batch_fn<uint8_t, kBatchNarrowBands>() : batch_fn<uint8_t, kBatchMaxBands>());
+    bool light = f32;
+    for (int i = 0; light && i < t.n; ++i) light = light_body(t.scenes[i].wavelet, t.scenes[i].bands);
+    const BatchFn k = light    ? batch_fn<float, kBatchLightBands>()
+                      : narrow ? (f32 ? batch_fn<float, kBatchNarrowBands>() : batch_fn<uint8_t, kBatchNarrowBands>())
+                               : (f32 ? batch_fn<float, kBatchMaxBands>() : batch_fn<uint8_t, kBatchMaxBands>());
     void *fn = k.fn;
     const int threads = k.threads, smem = k.smem;
     int occ = 0;
