@@ -393,11 +393,12 @@ int dwtfuse_set_band_chunks(int fwd, int bwd);
 /*
  * Store-path knob of the single-scene forward (a launch-shape choice, no
  * counterpart in the paper): with on = 1 (the default) dwtfuse_fuse takes the
- * staged kernel where it applies (a float output and whole 1024-column CTA
- * strips, the last one at least 7/8 full; rows on the 16-byte grid with at most
- * 6 bands, or other widths and more uint8 bands with a large output), which
- * writes the float rows through shared memory and bulk copies; with on = 0 it runs the warp-strip kernels everywhere.  The outputs
- * are the same bits either way.  Process-wide; other values are
+ * staged kernel where it applies (a float output, and at most 1/8 of its
+ * 1024-column strips' columns past the image; rows on the 16-byte grid with at
+ * most 6 bands, or other widths and more uint8 bands with a large output), which
+ * writes the float rows through shared memory and bulk copies; with on = 0 it
+ * runs the warp-strip kernels everywhere.  The outputs are the same bits either
+ * way.  Process-wide; other values are
  * DWTFUSE_EINVAL.
  */
 int dwtfuse_set_fuse_staging(int on);

@@ -372,9 +372,8 @@ __device__ __forceinline__ void idwt2_item(const DwtArgs &s, int64_t x0, int64_t
         load_coef3(Z + (H2 + mp) * W + W2, c, pair, G);
         d4_row_syn(L, G, rbp);
     }
-    // The next row's 12 coefficients are loaded one step ahead (the kernel
-    // runs two CTAs per SM at its register count either way), so a warp's
-    // loads overlap its arithmetic.
+    // The next row's 12 coefficients are loaded one step ahead (three CTAs per
+    // SM hold them), so a warp's loads overlap its arithmetic.
     float nL0[3], nG0[3], nL1[3], nG1[3];
     load_coef3(Z + m_s * W, c, pair, nL0);
     load_coef3(Z + m_s * W + W2, c, pair, nG0);
@@ -476,9 +475,9 @@ const void *dwt_staged_fn(bool f32) {
 // The staged forward: D4 (Haar's forward, two coefficient rows a step with
 // little arithmetic, measured slower staged: 16384^2 0.84 -> 0.74 of the copy
 // peak), coefficient rows on the 16-byte grid (the right quadrants start W/2
-// columns in, so W % 8 == 0) in a 16-byte-aligned plane, and a last
-// 1024-column strip at least 7/8 full (idle warps would wait at every step's
-// barrier).
+// columns in, so W % 8 == 0) in a 16-byte-aligned plane, and at most 1/8 of the
+// 1024-column strips' columns past the image (idle warps would wait at every
+// step's barrier).
 bool dwt_staged_applies(const DwtLaunch &d) {
     if (d.inverse || d.wavelet != DWTFUSE_D4 || d.W % 8 != 0 || (reinterpret_cast<uintptr_t>(d.dst_f32) & 15) != 0)
         return false;

@@ -47,7 +47,10 @@ extern __shared__ __align__(16) unsigned char batch_smem[];
 // copy (in the kernel's parameter block it would be read at run-time offsets
 // and its members held in registers).  A function of its own, not inlined:
 // each of an instance's bodies gets its own register allocation (all inlined
-// in one kernel they spilled up to 0.5 KB a thread).
+// in one kernel they spilled up to 0.5 KB a thread).  D4 bodies still report
+// spills, in bytes of stores a thread: uint8 12-44 up to 4 bands, 36-104 with 5-8,
+// float up to 12 and up to 52 (the kernels themselves 4-12; Haar none).  Not
+// measured: how many of them are registers saved for the caller, once an item.
 template <typename T, int WAV, int NB, int LAY, int MODE>
 static __device__ __noinline__ void batch_body(int x0, int m_s, int m_e) {
     const SceneArgs &s = *reinterpret_cast<const SceneArgs *>(batch_smem + (threadIdx.x >> 5) * kSceneBytes);

@@ -97,8 +97,8 @@ FwdFn fwd_kernel(const SceneArgs &s, int nb, int lay) {
 }  // namespace
 
 cudaError_t launch_fuse(const SceneArgs &s, int R, int blocks_per_sm, cudaStream_t stream) {
-    // Large scenes whose rows lie on the 16-byte grid with a float output: the
-    // staged kernel (its float rows go out as bulk copies).
+    // Scenes with a float output where it pays: the staged kernel (its float
+    // rows go out as bulk copies).
     if (fuse_staging() && fuse_staged_applies(s)) return launch_fuse_staged(s, R, stream);
     // Bands go in chunks of up to 8; the shifted-row instance (W % 4 == 2)
     // holds more live registers per band and takes balanced chunks of <= 6;

@@ -28,7 +28,8 @@
 //
 // A CTA that holds TMEM runs alone on its SM: up to 7 bands a CTA is 16 warps
 // (the SM's 64 K registers at 128 per thread), 8 bands 12 warps at up to 168
-// registers (at 128 the 8-band walker spills).  Against per-lane
+// registers.  Spills remain in D4 instances: 5-7 bands 16-60 bytes a thread, 8
+// bands 56 on aligned rows and none on the others.  Against per-lane
 // shared-memory slots for the sums (8-warp CTAs, two per SM): 16384^2 x 6
 // 1.525 -> 1.493 ms, 16384^2 x 7 2.212 -> 2.057 ms, 16382^2 x 8 2.805 ->
 // 2.554 ms.
@@ -66,7 +67,7 @@ struct FmLayout {
     // take 12.4 KB of shared memory per warp; 7-8 bands park 2.
     static constexpr int SR = NB <= 6 ? 4 : 2;
     // One CTA per SM (it holds TMEM): 16 warps at up to 128 registers, 8
-    // bands 12 warps at up to 168 (the 8-band walker spills at 128).
+    // bands 12 warps at up to 168 (16 warps ran 7-15 % slower).
     static constexpr int kThreads = NB <= 7 ? 512 : 384;
     static constexpr int kWarps = kThreads / 32;
     // Shifted rows of 5-7 bands, when every warp has an item: adjacent strips,
@@ -301,7 +302,7 @@ fuse_metrics_kernel(const __grid_constant__ SceneArgs s, double *partial, int st
         const int m_s = (int)(sy * R);
         const int m_e = (int)min((int64_t)m_s + R, s.H >> 1);
         const LaneCols c = lane_cols(x0, lane, s.W);
-            const int64_t x = x0 + 4 * lane;
+        const int64_t x = x0 + 4 * lane;
         const uint32_t keep = x + 4 <= s.W ? 0xffffffffu : (x + 2 <= s.W ? 0x0000ffffu : 0u);
         MetricEmit<NB, LAY> out{s,    c,     OutRun(s, c, 0, m_s), tile, rep, gsum, qs,
                                 se64, taddr, x0, m_s, m_e, lane, keep, true};

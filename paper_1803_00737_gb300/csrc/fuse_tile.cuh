@@ -777,7 +777,7 @@ struct OutRun {
 
 // Every lane writes its own 4 pixels to global memory.  kVec: 4-pixel
 // vectors; kShift: even rows as vectors (the lane at x = W-2 pairs), odd rows
-// through store4_shifted; kPairs: pixel pairs.
+// through the neighbour's pixels (store_f32, store_u8); kPairs: pixel pairs.
 // U8ONLY: the instance for a uint8 output alone.
 template <int LAY, int MODE, bool U8ONLY>
 struct DirectEmit {

@@ -10,8 +10,8 @@
 namespace dwtfuse {
 
 constexpr int kChunkBands = 8;     // bands per single-scene launch (more = several launches)
-constexpr int kBatchMaxBands = 8;
-constexpr int kBatchAltMaxBands = 6;  // bands of the batched shifted-row (W % 4 == 2) item body  // bands per scene in the batched kernel
+constexpr int kBatchMaxBands = 8;     // bands per scene in the batched kernel
+constexpr int kBatchAltMaxBands = 6;  // bands of the batched shifted-row (W % 4 == 2) item body
 constexpr int kMaxScenes = 128;    // scenes per batched launch
 constexpr int kDefaultRows = 32;   // most MS rows per warp work item of a batched launch by default
 constexpr size_t kQueueBytes = 16; // queue counter (8) + status word (4) + pad
@@ -139,9 +139,10 @@ constexpr int64_t kMetricPanPartialOffset = 8;
 cudaError_t launch_fuse_batched(BatchTable &t, unsigned long long *queue, int *status,
                                 int blocks_per_sm, cudaStream_t stream);
 
-// Staged single-scene forward (fuse_staged.cu): taken for rows on the 16-byte
-// grid with a float output, at most kStagedMaxBands bands, and a last CTA
-// strip at least 7/8 full.
+// Staged single-scene forward (fuse_staged.cu, which has the rule): a float
+// output and few idle columns in the CTA strips; rows on the 16-byte grid with at
+// most kStagedMaxBands bands at every size, shifted rows and more uint8 bands
+// where the output is large.
 bool fuse_staged_applies(const SceneArgs &s);
 cudaError_t launch_fuse_staged(const SceneArgs &s, int R, cudaStream_t stream);
 

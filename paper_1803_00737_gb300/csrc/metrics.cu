@@ -1520,11 +1520,11 @@ cudaError_t launch_metrics(const MetricLaunch &m, cudaStream_t stream) {
         e = fast_grid(fm, items, m.bands, &gm, true);
         if (e != cudaSuccess) return e;
         // The MS pass reads only MS and PAN.  When the kernel before it on the
-    // stream is the PAN-resolution pass or the fused forward + metrics kernel
-    // (ms_early), it is launched as that kernel's programmatic dependent: its
-    // CTAs start on SMs the primary has drained (the primary's last wave
-    // leaves SMs idle), and it waits for the primary grid only before it
-    // exits, so work after it still sees the primary's results.
+        // stream is the PAN-resolution pass or the fused forward + metrics kernel
+        // (ms_early), it is launched as that kernel's programmatic dependent: its
+        // CTAs start on SMs the primary has drained (the primary's last wave
+        // leaves SMs idle), and it waits for the primary grid only before it
+        // exits, so work after it still sees the primary's results.
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(gm);
         cfg.blockDim = dim3(fm.warps * 32);
