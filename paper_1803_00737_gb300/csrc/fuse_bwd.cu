@@ -482,7 +482,7 @@ BwdArgs make_bwd_args(const float *g, int bands, int64_t H, int64_t W, int wavel
 
 // MS rows per item of a batched launch over the scenes that it takes, by the
 // rule of balanced_rows on all their items together (8 x 1024^2 x 4: 64.9 ->
-// 48.9 us a call against 32 rows, 16 x 256^2 x 4: 50.6 -> 17.9).
+// 48.9 us a call against 32 rows, 16 x 256^2 x 4: 50.6 -> 15.4).
 template <class Takes>
 static int balanced_batch_rows(const BwdArgs *s, int n, Takes takes, int64_t warps) {
     static thread_local struct { int rows, strips; } group[kMaxScenes];  // neighbours of one height together

@@ -71,7 +71,7 @@ struct FmLayout {
     static constexpr int kThreads = NB <= 7 ? 512 : 384;
     static constexpr int kWarps = kThreads / 32;
     // Shifted rows of 5-7 bands, when every warp has an item: adjacent strips,
-    // which complete each other's sectors, in one CTA (8190^2 x 6 496 -> 462
+    // which complete each other's sectors, in one CTA (8190^2 x 6 496 -> 459
     // us, 11000 x 9998 x 6 857 -> 746, x 7 1022 -> 884, x 5 625 -> 613; not 3-4
     // bands, 493 -> 512, nor 8, 945 -> 966).  Which SM a warp's items run on
     // does not change its sums.
