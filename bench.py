@@ -89,8 +89,8 @@ KNOWN_TRAFFIC: dict[str, float] = {
     # read 689,644,885 + write 7,989,676,288 (mean of 3 launches)
     "22e4d6d25dce": 8679321173.0,
     # walkers with paired FP32 and running addresses, Q sums in two exact integers:
-    # read 706,280,533 + write 8,003,578,453 (mean of 3 launches)
-    "a8d6d23aba64": 8709858987.0,
+    # read 706,619,989 + write 8,003,330,901 (mean of 3 launches)
+    "2a4a99b2105c": 8709950890.0,
 }
 KERNEL_SOURCES = ("fuse_tile.cuh", "fuse_metrics.cu", "metric_q.cuh", "tmem.cuh")
 

@@ -52,11 +52,17 @@ struct QSum {
     long long hi = 0, lo = 0;
     __device__ __forceinline__ void add(float q) {
         const uint32_t w = __float_as_uint(q);
-        const int s = (int)((w >> 23) & 255u) - 73;  // q = +-m * 2^(s - 77)
-        if (s < 0) return;                           // 0
+        const int s = (int)((w >> 23) & 255u) - 73;  // q = +-m * 2^(s - 77); 0 where s <= -24
         const unsigned long long m = (w & 0x7fffffu) | 0x800000u;
-        const long long h = (long long)(s >= 45 ? m << (s - 45) : m >> (45 - s));
-        const long long l = s >= 45 ? 0ll : (long long)((m << s) & ((1ull << 45) - 1));
+        long long h = 0, l = 0;
+        if (s >= 45) {
+            h = (long long)(m << (s - 45));
+        } else if (s >= 0) {
+            h = (long long)(m >> (45 - s));
+            l = (long long)((m << s) & ((1ull << 45) - 1));
+        } else if (s > -24) {  // below 2^-54: what windows that nearly cancel leave (whole units of 2^-77)
+            l = (long long)(m >> -s);
+        }
         hi += (w >> 31) ? -h : h;
         lo += (w >> 31) ? -l : l;
     }
